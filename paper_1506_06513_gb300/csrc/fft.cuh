@@ -41,13 +41,29 @@ template <typename T, bool INV> struct Dft<T, 2, INV> {
     }
 };
 
+// i (p - q) for the inverse, -i (p - q) for the forward transform: the quarter
+// turn costs nothing when it is taken with the difference.
+template <bool INV, typename C> __device__ __forceinline__ C turned_sub(C p, C q)
+{
+    C r;
+    r.x = INV ? q.y - p.y : p.y - q.y;
+    r.y = INV ? p.x - q.x : q.x - p.x;
+    return r;
+}
+
+// x (c + i s) for the inverse, x (c - i s) for the forward transform
+template <bool INV, typename T> __device__ __forceinline__ cplx<T> turned(cplx<T> x, T c, T s)
+{
+    const cplx<T> m = cscale(x, c);
+    const T t = INV ? s : -s;
+    return mkc<T>(m.x - t * x.y, m.y + t * x.x);
+}
+
 template <typename T, bool INV> struct Dft<T, 4, INV> {
     __device__ __forceinline__ static void run(cplx<T>* v)
     {
         cplx<T> a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
-        cplx<T> a2 = cadd(v[1], v[3]);
-        cplx<T> d = csub(v[1], v[3]);
-        cplx<T> a3 = INV ? cmuli(d) : cmulmi(d);
+        cplx<T> a2 = cadd(v[1], v[3]), a3 = turned_sub<INV>(v[1], v[3]);
         v[0] = cadd(a0, a2);
         v[2] = csub(a0, a2);
         v[1] = cadd(a1, a3);
@@ -64,25 +80,26 @@ template <typename T, bool INV> struct Dft<T, 8, INV> {
         Dft<T, 4, INV>::run(e);
         Dft<T, 4, INV>::run(o);
         const T r = T(0.70710678118654752440084436210484903928);
-        // w8 = (1 -+ i)/sqrt2 ; w8^2 = -+i ; w8^3 = (-1 -+ i)/sqrt2
+        // w8 = (1 -+ i)/sqrt2 ; w8^2 = -+i ; w8^3 = (-1 -+ i)/sqrt2, the
+        // factor 1/sqrt2 taken with the sums below
         cplx<T> o1, o2, o3;
         if (INV) {
-            o1 = mkc<T>(r * (o[1].x - o[1].y), r * (o[1].x + o[1].y));
+            o1 = mkc<T>(o[1].x - o[1].y, o[1].x + o[1].y);
             o2 = cmuli(o[2]);
-            o3 = mkc<T>(-r * (o[3].x + o[3].y), r * (o[3].x - o[3].y));
+            o3 = mkc<T>(-o[3].x - o[3].y, o[3].x - o[3].y);
         } else {
-            o1 = mkc<T>(r * (o[1].x + o[1].y), r * (o[1].y - o[1].x));
+            o1 = mkc<T>(o[1].x + o[1].y, o[1].y - o[1].x);
             o2 = cmulmi(o[2]);
-            o3 = mkc<T>(r * (o[3].y - o[3].x), -r * (o[3].x + o[3].y));
+            o3 = mkc<T>(o[3].y - o[3].x, -o[3].x - o[3].y);
         }
         v[0] = cadd(e[0], o[0]);
         v[4] = csub(e[0], o[0]);
-        v[1] = cadd(e[1], o1);
-        v[5] = csub(e[1], o1);
+        v[1] = caxpy(r, o1, e[1]);
+        v[5] = caxpy(-r, o1, e[1]);
         v[2] = cadd(e[2], o2);
         v[6] = csub(e[2], o2);
-        v[3] = cadd(e[3], o3);
-        v[7] = csub(e[3], o3);
+        v[3] = caxpy(r, o3, e[3]);
+        v[7] = caxpy(-r, o3, e[3]);
     }
 };
 
@@ -103,19 +120,15 @@ template <typename T, bool INV> struct Dft<T, 16, INV> {
             for (int k1 = 0; k1 < 4; ++k1) y[n2][k1] = a[k1];
         }
         // y[n2][k1] *= w16^{n2 k1}; exponents 1, 2, 3, 2, 4, 6, 3, 6, 9
-        const T sg = INV ? T(1) : T(-1);
-        auto rot = [&](cplx<T> x, T c, T s) {   // x * (c + i sg s)
-            return mkc<T>(x.x * c - sg * x.y * s, x.y * c + sg * x.x * s);
-        };
-        y[1][1] = rot(y[1][1], c1, s1);
-        y[1][2] = rot(y[1][2], r, r);
-        y[1][3] = rot(y[1][3], s1, c1);
-        y[2][1] = rot(y[2][1], r, r);
+        y[1][1] = turned<INV, T>(y[1][1], c1, s1);
+        y[1][2] = turned<INV, T>(y[1][2], r, r);
+        y[1][3] = turned<INV, T>(y[1][3], s1, c1);
+        y[2][1] = turned<INV, T>(y[2][1], r, r);
         y[2][2] = INV ? cmuli(y[2][2]) : cmulmi(y[2][2]);
-        y[2][3] = rot(y[2][3], -r, r);
-        y[3][1] = rot(y[3][1], s1, c1);
-        y[3][2] = rot(y[3][2], -r, r);
-        y[3][3] = rot(y[3][3], -c1, -s1);
+        y[2][3] = turned<INV, T>(y[2][3], -r, r);
+        y[3][1] = turned<INV, T>(y[3][1], s1, c1);
+        y[3][2] = turned<INV, T>(y[3][2], -r, r);
+        y[3][3] = turned<INV, T>(y[3][3], -c1, -s1);
 #pragma unroll
         for (int k1 = 0; k1 < 4; ++k1) {
             cplx<T> a[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
@@ -131,13 +144,12 @@ template <typename T, bool INV> struct Dft<T, 3, INV> {
     {
         // w3 = -1/2 -+ i sqrt(3)/2
         const T s = T(0.86602540378443864676372317075293618347);
-        cplx<T> t1 = cadd(v[1], v[2]);
-        cplx<T> t2 = csub(v[0], cscale(t1, T(0.5)));
-        cplx<T> d = cscale(csub(v[1], v[2]), s);
-        cplx<T> t3 = INV ? cmuli(d) : cmulmi(d);
+        const cplx<T> t1 = cadd(v[1], v[2]);
+        const cplx<T> t2 = caxpy(T(-0.5), t1, v[0]);
+        const cplx<T> t3 = turned_sub<INV>(v[1], v[2]);
         v[0] = cadd(v[0], t1);
-        v[1] = cadd(t2, t3);
-        v[2] = csub(t2, t3);
+        v[1] = caxpy(s, t3, t2);
+        v[2] = caxpy(-s, t3, t2);
     }
 };
 
@@ -156,15 +168,11 @@ template <typename T, bool INV> struct Dft<T, 12, INV> {
             for (int k2 = 0; k2 < 4; ++k2) a[n1][k2] = b[k2];
         }
         // a[n1][k2] *= w12^{n1 k2}: exponents 1, 2, 3 (n1 = 1) and 2, 4, 6 (n1 = 2)
-        const T sg = INV ? T(1) : T(-1);
-        auto rot = [&](cplx<T> x, T cr, T si) {   // x * (cr + i sg si)
-            return mkc<T>(x.x * cr - sg * x.y * si, x.y * cr + sg * x.x * si);
-        };
-        a[1][1] = rot(a[1][1], c, h);
-        a[1][2] = rot(a[1][2], h, c);
+        a[1][1] = turned<INV, T>(a[1][1], c, h);
+        a[1][2] = turned<INV, T>(a[1][2], h, c);
         a[1][3] = INV ? cmuli(a[1][3]) : cmulmi(a[1][3]);
-        a[2][1] = rot(a[2][1], h, c);
-        a[2][2] = rot(a[2][2], -h, c);
+        a[2][1] = turned<INV, T>(a[2][1], h, c);
+        a[2][2] = turned<INV, T>(a[2][2], -h, c);
         a[2][3] = mkc<T>(-a[2][3].x, -a[2][3].y);
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) {
