@@ -567,6 +567,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
     constexpr int RB = sq_rows<L>();
     constexpr int NH = sq_nh<R, S>();
     using Map = SqMap<R, S>;
+    constexpr int NT = sq_kept<R, L>();    // line elements per lane that can be kept modes
     constexpr int CS = sq_slice<R, S>();   // line slice (S > 0: logical row R q + j at R q + (j ^ q))
     const int nx = g.nx, Mx = g.Mx, Mxp = g.Mxp;
     const int nrows = g.nz * g.ny;
@@ -577,8 +578,9 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
     FrameT<T>* Fs = reinterpret_cast<FrameT<T>*>(wacc + kWarpsX * 36);
     cplx<T>* twx = reinterpret_cast<cplx<T>*>(
         reinterpret_cast<unsigned char*>(Fs) + ((sizeof(FrameT<T>) + 15) / 16) * 16);
-    // w_nh^{j q} (q < R, j < L) at q L + (j ^ q): conflict-free both for a
-    // fixed q across lanes j and for a fixed j across lanes q
+    // w_nh^{j q} (q < R, j < L) at q L + j; with S = 2 at q L + (j ^ q):
+    // conflict-free both for a fixed q across lanes j and for a fixed j across
+    // lanes q (only the forward pass of lane pairs reads the latter)
     cplx<T>* tw2 = twx + NH;
     cplx<T>* buf = tw2 + NH;               // C line slices of CS values
     __shared__ int rowmask[RB];
@@ -598,7 +600,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
     for (int i = tid; i < NH; i += blockDim.x) twx[i] = twv(i);
     for (int i = tid; i < NH; i += blockDim.x) {
         const int q = i / L, jj = i % L;
-        tw2[q * L + (S == 0 ? jj : (jj ^ q))] = twv((2 * jj * q) % nx);
+        tw2[q * L + (S == 2 ? (jj ^ q) : jj)] = twv((2 * jj * q) % nx);
     }
     load_frame_t<T>(Fs, ex.frame);
 
@@ -654,7 +656,8 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
 #pragma unroll
             for (int t = 0; t < R; ++t) {
                 const int k = j + L * t;
-                v[t] = (r < nrows && k < Mx) ? src[k] : mkc<T>(0, 0);
+                if (t < NT) v[t] = (r < nrows && k < Mx) ? src[k] : mkc<T>(0, 0);
+                else v[t] = mkc<T>(0, 0);   // dropped by the 2/3 rule whatever j is
             }
             if (j == 0) v[0].y = T(0);     // a real line has a real mean
             // ---- inverse: c2r pre-processing, radix R over t and the twiddles
@@ -662,7 +665,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
             sq_exchange_pre<T, R, L>(v, j, twx);
             Dft<T, R, true>::run(v);
 #pragma unroll
-            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], cconj(tw2[q * L + (S == 0 ? j : (j ^ q))]));
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], cconj(tw2[q * L + (S == 2 ? (j ^ q) : j)]));
             if constexpr (S == 0) {
                 // Y[j][n1] at n1 L + (j ^ n1 % L); lane j then takes n1 = j + L m
 #pragma unroll
@@ -730,38 +733,38 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
         if constexpr (sizeof(T) == 4 && (sq_wide<T, R, S>() || S == 0) && !SPONGE && !LAYER) {
             constexpr int NH2 = NH / 2;
             const int items = RB * NH2;
-            T e_tile = T(0);
+            float2 e2 = make_float2(0.0f, 0.0f);
             for (int it = 0; it < (items + 191) / 192; ++it) {
                 const int i = tid + it * 192;
                 const int rr = i / NH2, lrow = 2 * (i % NH2);
                 if (i < items && row0 + rr < nrows) {
                     const int slot = sq_line_slot<T, R, S>(lrow);   // even; row lrow + 1 at slot + 1
-                    float4 uq[3], wq[3];
+                    // two packed pairs (points 2p, 2p + 1) per component
+                    float2 u[2][3], w[2][3];
 #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        uq[q] = *reinterpret_cast<const float4*>(buf + (q * RB + rr) * CS + slot);
-                        wq[q] = *reinterpret_cast<const float4*>(buf + ((3 + q) * RB + rr) * CS + slot);
+                        const float4 a = *reinterpret_cast<const float4*>(buf + (q * RB + rr) * CS + slot);
+                        const float4 b = *reinterpret_cast<const float4*>(buf + ((3 + q) * RB + rr) * CS + slot);
+                        u[0][q] = make_float2(a.x, a.y);
+                        u[1][q] = make_float2(a.z, a.w);
+                        w[0][q] = make_float2(b.x, b.y);
+                        w[1][q] = make_float2(b.z, b.w);
                     }
-                    T nl[4][3];
+                    float2 nl[2][3];
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        T u[3], om[3];
-#pragma unroll
-                        for (int q = 0; q < 3; ++q) {
-                            u[q] = h == 0 ? uq[q].x : h == 1 ? uq[q].y : h == 2 ? uq[q].z : uq[q].w;
-                            om[q] = h == 0 ? wq[q].x : h == 1 ? wq[q].y : h == 2 ? wq[q].z : wq[q].w;
-                        }
-                        cross3(u, om, nl[h]);
-                        const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-                        e_tile += uu;
-                        m_acc = fmax(m_acc, uu);
+                    for (int h = 0; h < 2; ++h) {
+                        cross3_pair(u[h], w[h], nl[h]);
+                        const float2 uu = __ffma2_rn(u[h][2], u[h][2], __ffma2_rn(u[h][1], u[h][1], __fmul2_rn(u[h][0], u[h][0])));
+                        e2 = __fadd2_rn(e2, uu);
+                        m_acc = fmaxf(m_acc, fmaxf(uu.x, uu.y));
                     }
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
                         *reinterpret_cast<float4*>(buf + ((3 + q) * RB + rr) * CS + slot) =
-                            make_float4(nl[0][q], nl[1][q], nl[2][q], nl[3][q]);
+                            make_float4(nl[0][q].x, nl[0][q].y, nl[1][q].x, nl[1][q].y);
                 }
             }
+            const T e_tile = e2.x + e2.y;
             e_acc += double(e_tile);
             if (!isfinite(e_tile)) bad = 1;
         } else {
@@ -931,7 +934,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
 #pragma unroll
                 for (int t = 0; t < R; ++t) v[t] = line[R * t + (j ^ sq_swz<T, R, S>(t))];
 #pragma unroll
-                for (int t = 1; t < R; ++t) v[t] = cmul(v[t], tw2[t * R + (j ^ t)]);
+                for (int t = 1; t < R; ++t) v[t] = cmul(v[t], tw2[t * R + j]);
             } else {
                 // lane j = (k1, p): radix 2 over the two halves h of its points
                 // k1 + R k' + R^2 h, the twiddles w_2R^{p k'}, radix R over k',
@@ -962,24 +965,24 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
             cplx<T>* out = W + ((size_t)fld * nrows + (r < nrows ? r : 0)) * Mxp;
 #pragma unroll
             for (int s2 = 0; s2 < R / 2; ++s2) {
-                cplx<T> a, b;   // partner's Z[s2] and Z[R-1-s2]
-                a.x = __shfl_sync(0xffffffffu, v[s2].x, (L - j) & (L - 1), L);
-                a.y = __shfl_sync(0xffffffffu, v[s2].y, (L - j) & (L - 1), L);
-                b.x = __shfl_sync(0xffffffffu, v[R - 1 - s2].x, (L - j) & (L - 1), L);
-                b.y = __shfl_sync(0xffffffffu, v[R - 1 - s2].y, (L - j) & (L - 1), L);
+                // elements q1 = s2 and, where it can be a kept mode, q2 = R-1-s2
+                const int q1 = s2, q2 = R - 1 - s2;
+                cplx<T> a = mkc<T>(0, 0), b;   // partner's Z[s2] and Z[R-1-s2]
+                b.x = __shfl_sync(0xffffffffu, v[q2].x, (L - j) & (L - 1), L);
+                b.y = __shfl_sync(0xffffffffu, v[q2].y, (L - j) & (L - 1), L);
+                if (q2 < NT) {
+                    a.x = __shfl_sync(0xffffffffu, v[q1].x, (L - j) & (L - 1), L);
+                    a.y = __shfl_sync(0xffffffffu, v[q1].y, (L - j) & (L - 1), L);
+                }
                 if (r < nrows) {
-                    const int q1 = s2, q2 = R - 1 - s2;
                     const int k1 = j + L * q1, k2 = j + L * q2;
-                    cplx<T> m1, m2;
-                    if (j != 0) {
-                        m1 = b;    // Z[nh - k1] = partner's Z[R-1-q1]
-                        m2 = a;
-                    } else {
-                        m1 = v[(R - q1) % R];
-                        m2 = v[(R - q2) % R];
-                    }
+                    // Z[nh - k]: the partner's mirror element, lane 0's own
+                    const cplx<T> m1 = j != 0 ? b : v[(R - q1) % R];
                     if (k1 < Mxp) out[k1] = k1 < Mx ? r2c_post<T>(v[q1], m1, twx[k1]) : mkc<T>(0, 0);
-                    if (k2 < Mxp) out[k2] = k2 < Mx ? r2c_post<T>(v[q2], m2, twx[k2]) : mkc<T>(0, 0);
+                    if (q2 < NT) {
+                        const cplx<T> m2 = j != 0 ? a : v[(R - q2) % R];
+                        if (k2 < Mxp) out[k2] = k2 < Mx ? r2c_post<T>(v[q2], m2, twx[k2]) : mkc<T>(0, 0);
+                    }
                 }
             }
         }

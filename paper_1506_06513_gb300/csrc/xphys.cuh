@@ -166,6 +166,16 @@ __device__ __forceinline__ void cross3(const T* a, const T* b, T* c)
     c[2] = a[0] * b[1] - a[1] * b[0];
 }
 
+// u x w of two points at once (packed pairs), rounded as cross3 rounds it
+__device__ __forceinline__ void cross3_pair(const float2* u, const float2* w, float2* c)
+{
+    const float2 minus = make_float2(-1.0f, -1.0f);
+    const float2 v[3] = {__fmul2_rn(w[0], minus), __fmul2_rn(w[1], minus), __fmul2_rn(w[2], minus)};
+    c[0] = __ffma2_rn(u[1], w[2], __fmul2_rn(u[2], v[1]));
+    c[1] = __ffma2_rn(u[2], w[0], __fmul2_rn(u[0], v[2]));
+    c[2] = __ffma2_rn(u[0], w[1], __fmul2_rn(u[1], v[0]));
+}
+
 // Mask, colour (0 fluid, 1 body, 2/3 wings) and solid velocity at X.
 template <typename T>
 __device__ __forceinline__ void solid_at(const FrameT<T>& F, const T* X, const bool* inrow, T& chi,
@@ -269,6 +279,24 @@ __device__ __forceinline__ cplx<T> r2c_post(cplx<T> Zk, cplx<T> Zm, cplx<T> wk)
     return mkc<T>(T(0.5) * fmadd(wk.y, bx, fmadd(wk.x, by, ax)), T(0.5) * fmadd(-wk.x, bx, fmadd(wk.y, by, ay)));
 }
 
+// c2r pre-processing with X[nh - k] = 0 (a mode that the 2/3 rule drops): the
+// same value as c2r_pre(Xk, 0, wk) in half the operations.
+template <typename T>
+__device__ __forceinline__ cplx<T> c2r_pre_nomirror(cplx<T> Xk, cplx<T> wk)
+{
+    return mkc<T>(fmadd(Xk.x, wk.y, fmadd(-Xk.y, wk.x, Xk.x)), fmadd(Xk.y, wk.y, fmadd(Xk.x, wk.x, Xk.y)));
+}
+// ... and with X[k] = 0.
+template <typename T>
+__device__ __forceinline__ cplx<T> c2r_pre_dropped(cplx<T> Xm, cplx<T> wk)
+{
+    return mkc<T>(fmadd(-Xm.x, wk.y, fmadd(-Xm.y, wk.x, Xm.x)), fmadd(Xm.y, wk.y, fmadd(-Xm.x, wk.x, -Xm.y)));
+}
+
+// Registers t of a lane's line elements k = j + L t, t < R = nh / L, that can
+// hold a mode kept by the 2/3 rule (k <= nx/3 = 2 nh / 3); the others are zero.
+template <int R, int L> constexpr int sq_kept() { return (2 * R * L / 3) / L + 1; }
+
 template <typename T, int R, int L>
 __device__ __forceinline__ void sq_exchange_pre(cplx<T>* x, int j, const cplx<T>* twx)
 {
@@ -279,22 +307,30 @@ __device__ __forceinline__ void sq_exchange_pre(cplx<T>* x, int j, const cplx<T>
     // where the other lanes send elements s and R-1-s.  The pairs (s, R-1-s)
     // go from the middle outwards, so every element read is still unmodified
     // (element s+1 was overwritten the iteration before: carried from there).
+    // Elements t >= NT hold dropped modes on every lane: nothing is exchanged
+    // for them.
+    constexpr int NT = sq_kept<R, L>();
     const int partner = (L - j) & (L - 1);
     const bool self = j == 0;
     cplx<T> carry = x[R / 2];   // the original element s + 1
 #pragma unroll
     for (int s = R / 2 - 1; s >= 0; --s) {
         const cplx<T> xs = x[s], xt = x[R - 1 - s];
-        const cplx<T> up = s == 0 ? mkc<T>(0, 0) : x[s == 0 ? 0 : R - s];
         const cplx<T> sa = self ? carry : xs;   // mirror of element R-1-s
-        const cplx<T> sb = self ? up : xt;      // mirror of element s
         cplx<T> a, b;
         a.x = __shfl_sync(0xffffffffu, sa.x, partner, L);
         a.y = __shfl_sync(0xffffffffu, sa.y, partner, L);
-        b.x = __shfl_sync(0xffffffffu, sb.x, partner, L);
-        b.y = __shfl_sync(0xffffffffu, sb.y, partner, L);
-        x[s] = c2r_pre<T>(xs, b, twx[j + L * s]);
-        x[R - 1 - s] = c2r_pre<T>(xt, a, twx[j + L * (R - 1 - s)]);
+        if (R - 1 - s < NT) {
+            const cplx<T> up = s == 0 ? mkc<T>(0, 0) : x[s == 0 ? 0 : R - s];
+            const cplx<T> sb = self ? up : xt;      // mirror of element s
+            b.x = __shfl_sync(0xffffffffu, sb.x, partner, L);
+            b.y = __shfl_sync(0xffffffffu, sb.y, partner, L);
+            x[s] = c2r_pre<T>(xs, b, twx[j + L * s]);
+            x[R - 1 - s] = c2r_pre<T>(xt, a, twx[j + L * (R - 1 - s)]);
+        } else {
+            x[s] = c2r_pre_nomirror<T>(xs, twx[j + L * s]);
+            x[R - 1 - s] = c2r_pre_dropped<T>(a, twx[j + L * (R - 1 - s)]);
+        }
         carry = xs;
     }
 }
