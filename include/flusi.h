@@ -342,7 +342,8 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * for y; columns of the flattened (y, x) plane for z), a power of two of at
  * least 32 bytes of complex values (4 in FP32, 2 in FP64) and at most 256.
  * x_kernel: 0 (default) the register-resident line kernel where one exists
- * (nx = 128, 256, 512, 1024, and its rectangular form at nx = 64, 96), 1 the
+ * (nx = 128, 256, 512, 1024, and its rectangular form at nx = 64, 96; in FP32
+ * the general line kernels at every other length from 16 on), 1 the
  * shared-memory kernel of every length.
  * y_pair: 1 the y passes' paired kernel, a cluster of two CTAs per tile,
  * each holding the grid rows of one parity and transforming them at half the
@@ -352,7 +353,8 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  *
  * flusi_get_tuning fills every field, including the read-only ones: the
  * radices each pass takes (0-terminated), the columns a tile takes, and
- * whether the x pass runs the register-resident kernel.
+ * whether the x pass runs the register-resident kernel that also forms the
+ * sponge term (1 at the six lengths named first, 0 for the general kernels).
  * flusi_set_tuning takes the six settings (the rest is ignored); any
  * other value is FLUSI_EINVAL with nothing changed.  On a bound handle it
  * waits for the handle's stream, uploads the new digit-reversal tables and

@@ -18,6 +18,8 @@
 // (P = blockDim / C threads per column).
 #pragma once
 
+#include <utility>
+
 #include "common.cuh"
 
 namespace flusi {
@@ -183,6 +185,82 @@ template <typename T, bool INV> struct Dft<T, 12, INV> {
         }
     }
 };
+
+// cos(2 pi k / n) and sin(2 pi k / n) at compile time: the angle folded into
+// [0, pi/4] by the symmetries of the circle, then the Taylor series (its first
+// dropped term is below 1e-22 there).
+constexpr double taylor_cos(double x, int first)
+{
+    // sum of (-1)^m x^(2m + first) / (2m + first)!, first = 0 (cos) or 1 (sin)
+    double term = first ? x : 1.0, sum = term;
+    for (int i = 1; i < 11; ++i) {
+        term *= -x * x / double((2 * i + first) * (2 * i + first - 1));
+        sum += term;
+    }
+    return sum;
+}
+constexpr double cos_turn(int k, int n)
+{
+    constexpr double two_pi = 6.283185307179586476925286766559;
+    k = (k % n + n) % n;
+    if (2 * k > n) k = n - k;                          // cos(-a) = cos(a)
+    const bool back = 4 * k > n;                       // cos(pi - a) = -cos(a)
+    const int m = back ? n - 2 * k : 2 * k;            // angle 2 pi m / (2 n), in [0, pi/2]
+    const double c = 4 * m > n ? taylor_cos(two_pi * (n - 2 * m) / (4.0 * n), 1)   // sin(pi/2 - a)
+                               : taylor_cos(two_pi * m / (2.0 * n), 0);
+    return back ? -c : c;
+}
+constexpr double sin_turn(int k, int n) { return cos_turn(4 * k - n, 4 * n); }
+
+// x w with w = exp(2 pi i E / N) for the inverse, its conjugate for the forward transform
+template <typename T, int E, int N, bool INV> __device__ __forceinline__ cplx<T> turned_by(cplx<T> x)
+{
+    constexpr int e = E % N;
+    if constexpr (e == 0) return x;
+    else if constexpr (2 * e == N) return mkc<T>(-x.x, -x.y);
+    else if constexpr (4 * e == N) return INV ? cmuli(x) : cmulmi(x);
+    else if constexpr (4 * e == 3 * N) return INV ? cmulmi(x) : cmuli(x);
+    else {
+        constexpr T c = T(cos_turn(e, N)), s = T(sin_turn(e, N));
+        return turned<INV, T>(x, c, s);
+    }
+}
+
+// N = A B point DFT: with n = B a + b and k = k1 + A k2,
+// X[k1 + A k2] = sum_b w_B^{b k2} w_N^{b k1} (sum_a x[B a + b] w_A^{a k1}).
+template <typename T, int A, int B, bool INV> struct DftProduct {
+    template <size_t... I>
+    __device__ __forceinline__ static void turn(cplx<T> (*y)[A], std::index_sequence<I...>)
+    {
+        ((y[I / A][I % A] = turned_by<T, int((I / A) * (I % A)), A * B, INV>(y[I / A][I % A])), ...);
+    }
+    __device__ __forceinline__ static void run(cplx<T>* v)
+    {
+        cplx<T> y[B][A];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+#pragma unroll
+            for (int a = 0; a < A; ++a) y[b][a] = v[B * a + b];
+            Dft<T, A, INV>::run(y[b]);
+        }
+        turn(y, std::make_index_sequence<A * B>());
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            cplx<T> t[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) t[b] = y[b][k1];
+            Dft<T, B, INV>::run(t);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = t[k2];
+        }
+    }
+};
+template <typename T, bool INV> struct Dft<T, 6, INV> : DftProduct<T, 2, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 9, INV> : DftProduct<T, 3, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 18, INV> : DftProduct<T, 2, 9, INV> {};
+template <typename T, bool INV> struct Dft<T, 24, INV> : DftProduct<T, 8, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 27, INV> : DftProduct<T, 3, 9, INV> {};
+template <typename T, bool INV> struct Dft<T, 32, INV> : DftProduct<T, 8, 4, INV> {};
 
 // v[t] *= w^(k t) for t = 1..R-1 from the table (conjugated for the inverse):
 // tw[k * step] holds w^k.

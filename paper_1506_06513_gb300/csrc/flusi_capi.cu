@@ -1335,7 +1335,7 @@ int flusi_autotune(flusi_t h, int steps, const char* cache_path, flusi_tuning* o
             for (int i = 0; i < FLUSI_MAX_STAGES; ++i)
                 sig += std::to_string(got.y_radix[i]) + "," + std::to_string(got.zf_radix[i]) + ",";
             sig += std::to_string(got.y_tile_cols) + "," + std::to_string(got.z_tile_cols) + "," +
-                   std::to_string(got.x_line_kernel) + "," + std::to_string(got.y_paired);
+                   std::to_string(xpass_kernel(h->prec == FLUSI_FP64, h->g)) + "," + std::to_string(got.y_paired);
             if (std::find(seen.begin(), seen.end(), sig) != seen.end()) continue;
             seen.push_back(sig);
             double ms = 0;

@@ -23,11 +23,44 @@
 
 #include "fft.cuh"
 #include "kernels.cuh"
+#include "xline.cuh"
 #include "xphys.cuh"
 
 namespace flusi {
 
+const XLineOps* xline_table_small(int* n);
+const XLineOps* xline_table_medium(int* n);
+const XLineOps* xline_table_large(int* n);
+const XLineOps* xline_table_huge(int* n);
+
 namespace {
+
+// The line kernels of this FP32 grid (xline.cuh): any length from 16 on, unless
+// the shared-memory kernels are asked for.
+template <class F> void each_xline(F f)
+{
+    for (auto table : {xline_table_small, xline_table_medium, xline_table_large, xline_table_huge}) {
+        int n = 0;
+        const XLineOps* t = table(&n);
+        for (int i = 0; i < n; ++i) f(t[i]);
+    }
+}
+template <typename T> const XLineOps* xline_of(const Geom& g)
+{
+    const XLineOps* found = nullptr;
+    if (sizeof(T) == 4 && !g.xgeneric)
+        each_xline([&](const XLineOps& o) {
+            if (o.nx == g.nx) found = &o;
+        });
+    return found;
+}
+int sm_count_here()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
 
 constexpr int kThreadsX = 192;
 constexpr int kWarpsX = kThreadsX / 32;
@@ -1102,12 +1135,10 @@ template <typename T> size_t x_smem(const Geom& g, int lgRB, int NF)
 
 template <typename T> int x_grid(const Geom& g)
 {
-    int dev = 0, sm_count = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-    if (sm_count <= 0) sm_count = 1;
+    const int sm_count = sm_count_here();
     int per_sm = 0, ntiles = 0;
     const int kind = sq_kind<T>(g);
+    const XLineOps* line = kind == 0 ? xline_of<T>(g) : nullptr;
 #define FLUSI_SQ_OCC(R, S)                                                                          \
     ntiles = ceil_div(g.nz * g.ny, sq_rows<sq_lanes<R, S>()>());                                               \
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, false>, 192, \
@@ -1124,6 +1155,9 @@ template <typename T> int x_grid(const Geom& g)
         FLUSI_SQ_OCC(12, 0)
     } else if (kind == 80) {
         FLUSI_SQ_OCC(8, 0)
+    } else if (line) {
+        ntiles = ceil_div(g.nz * g.ny, line->rows);
+        per_sm = line->phys_per_sm();
     } else {
         const int lg = x_lgrb<T>(g);
         ntiles = ceil_div(g.nz * g.ny, 1 << lg);
@@ -1150,6 +1184,23 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
     cplx<T>* w = (cplx<T>*)W;
     const bool layer = ex.layer0[0] < g.nx || ex.layer0[1] < g.ny || ex.layer0[2] < g.nz;
     const bool sponge = ex.sponge_fused != 0;
+    if constexpr (sizeof(T) == 4) {
+        const XLineOps* line = xline_of<T>(g);
+        if (line && (mode == XP_R2C || mode == XP_C2R || mode == XP_SPONGE)) {
+            line->lines(mode, s, w, g, tw, ex, sm_count_here());
+            return cudaGetLastError();
+        }
+        if (line && line->phys && mode == XP_PHYS && sq_kind<T>(g) == 0) {
+            const Batch& B = current_batch();
+            XExtra e = ex;
+            e.nvirt = x_grid<T>(g);
+            // a batch of n members runs about one resident wave in all (launch_sq)
+            const int resident = sm_count_here() * std::max(1, line->phys_per_sm());
+            const int run = B.n > 1 ? std::min(e.nvirt, std::max(1, ceil_div(resident, B.n))) : e.nvirt;
+            line->phys(dim3(run, 1, B.n), s, w, g, tw, e, st, B.mb);
+            return cudaGetLastError();
+        }
+    }
     switch (mode) {
     case XP_PHYS:
         switch (sq_kind<T>(g)) {
@@ -1195,6 +1246,12 @@ int xpass_fuses_sponge(int fp64, const Geom& g)
     return fp64 ? sq_kind<double>(g) != 0 : sq_kind<float>(g) != 0;
 }
 
+int xpass_kernel(int fp64, const Geom& g)
+{
+    if (fp64 ? sq_kind<double>(g) != 0 : sq_kind<float>(g) != 0) return 1;
+    return !fp64 && xline_of<float>(g) ? 2 : 0;
+}
+
 cudaError_t launch_xpass(int fp64, int mode, void* W, const Geom& g, const FftPlan& plan,
                          const double2* tw, const int* pos, const XExtra& ex, const StepState* st,
                          cudaStream_t s)
@@ -1210,7 +1267,11 @@ cudaError_t launch_xpass(int fp64, int mode, void* W, const Geom& g, const FftPl
 cudaError_t configure_xpass()
 {
     const int big = 200 * 1024;
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
+    each_xline([&](const XLineOps& o) {
+        if (!e) e = o.configure();
+    });
+    if (e) return e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
     FLUSI_SMEM((k_xpass<float, XP_PHYS>))
