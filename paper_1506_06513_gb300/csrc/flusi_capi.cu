@@ -371,31 +371,32 @@ cudaError_t enqueue_step(flusi_t h, cudaStream_t s, cudaEvent_t* ev, const char*
         if (names) names[k] = next;
         ++k;
     };
-    // Without per-kernel events the two single-block kernels of the first
-    // right-hand side run on the side stream: the kinematics only have to
-    // finish before the x pass, the scalars (dt, coefficients, force row) only
-    // before the update.
+    // Without per-kernel events the small kernels run on the side stream: a
+    // right-hand side's kinematics only have to finish before its x pass (and
+    // start after the x pass before, which reads the frame they overwrite), the
+    // scalars (dt, coefficients, force row) only before the first update.
     const bool branch = ev == nullptr;
     cudaStream_t sk = branch ? h->side : s;
     const int nfwd = has_sponge(h) ? 6 : 3;
     const int stages = is_rk4(h) ? 4 : 1;
     const double frac[4] = {0.0, 0.5, 0.5, 1.0};
+    auto kinematics = [&](int q) {
+        k_kinematics<<<dim3(1, 1, current_batch().n), 32, 0, sk>>>(
+            at<flusi_insect>(h, h->oins), st, coef, at<Frame>(h, h->oframe), box_margin(h), frac[q],
+            current_batch().mb, make_shape(h), 1, 1.0 / g.eta);
+        const cudaError_t err = cudaGetLastError();
+        return err || !branch ? err : cudaEventRecord(h->ev_kin, sk);
+    };
     for (int q = 0; q < stages; ++q) {
         const char* const* nm = kStageNames[q];
         // the right-hand side at the stage state: u^n first, then the RK4 stage buffer
         void* ustage = q == 0 ? h->ws + h->oU : h->ws + h->oUt;
-        cudaStream_t skq = q == 0 ? sk : s;
-        const bool br = branch && q == 0;
         mark(nm[0]);
-        if (br) {
+        if (branch && q == 0) {
             if ((e = cudaEventRecord(h->ev_fork, s))) return e;
             if ((e = cudaStreamWaitEvent(sk, h->ev_fork, 0))) return e;
         }
-        k_kinematics<<<dim3(1, 1, current_batch().n), 32, 0, skq>>>(
-            at<flusi_insect>(h, h->oins), st, coef, at<Frame>(h, h->oframe), box_margin(h), frac[q],
-            current_batch().mb, make_shape(h), 1, 1.0 / g.eta);
-        if ((e = cudaGetLastError())) return e;
-        if (br && (e = cudaEventRecord(h->ev_kin, sk))) return e;
+        if ((!branch || q == 0) && (e = kinematics(q))) return e;
         mark(nm[1]);
         const CUtensorMap* umap = q == 0 ? &h->zmaps.u : &h->zmaps.ut;
         const int ubh = q == 0 ? h->zmaps.u_bh : h->zmaps.ut_bh;
@@ -404,7 +405,7 @@ cudaError_t enqueue_step(flusi_t h, cudaStream_t s, cudaEvent_t* ev, const char*
         mark(nm[2]);
         if ((e = launch_ypass(fp64, true, W, g, h->py, ty, at<int>(h, h->opy), 6, st, &h->ymaps, &st->status, s, &h->pyh, at<int>(h, h->opyh)))) return e;
         mark(g.xtc ? kTcNames[q] : nm[3]);
-        if (br && (e = cudaStreamWaitEvent(s, h->ev_kin, 0))) return e;
+        if (branch && (e = cudaStreamWaitEvent(s, h->ev_kin, 0))) return e;
         XExtra xe{};
         xe.frame = at<Frame>(h, h->oframe);
         xe.shape = make_shape(h);
@@ -414,12 +415,12 @@ cudaError_t enqueue_step(flusi_t h, cudaStream_t s, cudaEvent_t* ev, const char*
         xe.sponge_fused = has_sponge(h) && !sponge_kernel(h);
         xe.err = &st->status;
         if ((e = launch_xpass(fp64, XP_PHYS, W, g, h->px, tx, at<int>(h, h->opx), xe, st, s))) return e;
+        if (branch) {
+            if ((e = cudaEventRecord(h->ev_x, s))) return e;
+            if ((e = cudaStreamWaitEvent(sk, h->ev_x, 0))) return e;
+        }
         if (q == 0) {
             mark("scalars");
-            if (branch) {
-                if ((e = cudaEventRecord(h->ev_x, s))) return e;
-                if ((e = cudaStreamWaitEvent(sk, h->ev_x, 0))) return e;
-            }
             double3 opts = make_double3(h->opt.cfl, h->opt.dt_fixed, h->opt.dt_max);
             k_scalars<<<dim3(1, 1, current_batch().n), 256, 0, sk>>>(g, at<double>(h, h->opart), h->xgrid, st, coef, at<double>(h, h->orows),
                                          h->opt.force_ring, at<double>(h, h->oetab), opts, rk4_dt_diff(h),
@@ -427,6 +428,7 @@ cudaError_t enqueue_step(flusi_t h, cudaStream_t s, cudaEvent_t* ev, const char*
             if ((e = cudaGetLastError())) return e;
             if (branch && (e = cudaEventRecord(h->ev_sc, sk))) return e;
         }
+        if (branch && q + 1 < stages && (e = kinematics(q + 1))) return e;
         if (sponge_kernel(h)) {
             mark(nm[4]);
             // chi_sp omega of the vorticity still in W[3..5] (x transformed back in place)

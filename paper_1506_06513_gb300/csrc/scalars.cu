@@ -18,38 +18,6 @@ struct M3 {
     double a[9];
 };
 
-__device__ M3 rot_x(double xi)
-{
-    double c = cos(xi), s = sin(xi);
-    return {{1, 0, 0, 0, c, s, 0, -s, c}};
-}
-__device__ M3 rot_y(double xi)
-{
-    double c = cos(xi), s = sin(xi);
-    return {{c, 0, -s, 0, 1, 0, s, 0, c}};
-}
-__device__ M3 rot_z(double xi)
-{
-    double c = cos(xi), s = sin(xi);
-    return {{c, s, 0, -s, c, 0, 0, 0, 1}};
-}
-__device__ M3 mul(const M3& A, const M3& B)
-{
-    M3 C;
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
-            C.a[i * 3 + j] = A.a[i * 3] * B.a[j] + A.a[i * 3 + 1] * B.a[3 + j] + A.a[i * 3 + 2] * B.a[6 + j];
-    return C;
-}
-// A^T x (the inverse of a rotation applied to x)
-__device__ void apply_t(const M3& A, const double* x, double* y)
-{
-    double t0 = A.a[0] * x[0] + A.a[3] * x[1] + A.a[6] * x[2];
-    double t1 = A.a[1] * x[0] + A.a[4] * x[1] + A.a[7] * x[2];
-    double t2 = A.a[2] * x[0] + A.a[5] * x[1] + A.a[8] * x[2];
-    y[0] = t0, y[1] = t1, y[2] = t2;
-}
-
 // A x
 __device__ void apply(const M3& A, const double* x, double* y)
 {
@@ -67,27 +35,6 @@ __device__ void cross3(const double* a, const double* b, double* c)
     c[0] = c0, c[1] = c1, c[2] = c2;
 }
 
-// a0/2 + sum a_i cos(2 pi i f t) + b_i sin(2 pi i f t) and its first two time
-// derivatives
-__device__ void series(double a0, const double* a, const double* b, int nf, double f, double t,
-                       double* v, double* dv, double* ddv)
-{
-    const double two_pi = 6.283185307179586476925286766559;
-    double s = 0.5 * a0, d = 0.0, dd = 0.0;
-    for (int i = 0; i < nf; ++i) {
-        double w = two_pi * (i + 1) * f;
-        double sn, cs;
-        sincos(w * t, &sn, &cs);
-        const double c = a[i] * cs + b[i] * sn;
-        s += c;
-        d += w * (b[i] * cs - a[i] * sn);
-        dd -= w * w * c;
-    }
-    *v = s;
-    *dv = d;
-    *ddv = dd;
-}
-
 // Body-to-global matrix of the quaternion (e0, e1, e2, e3) as printed in
 // Sec. 3.6; its transpose is the global-to-body matrix M_body.
 __device__ M3 quat_to_global(const double* e)
@@ -96,14 +43,6 @@ __device__ M3 quat_to_global(const double* e)
     return {{a * a + b * b - c * c - d * d, 2 * (b * c - a * d), 2 * (b * d + a * c),
              2 * (b * c + a * d), a * a - b * b + c * c - d * d, 2 * (c * d - a * b),
              2 * (b * d - a * c), 2 * (c * d + a * b), a * a - b * b - c * c + d * d}};
-}
-
-__device__ void box_grow(double* box, const double* p)
-{
-    for (int i = 0; i < 3; ++i) {
-        box[2 * i] = fmin(box[2 * i], p[i]);
-        box[2 * i + 1] = fmax(box[2 * i + 1], p[i]);
-    }
 }
 
 // Free flight (Sec. 3.6, Eq. oh_my_god_look_a_vector): one AB2 step of the
@@ -171,13 +110,291 @@ __device__ void advance_body(flusi_insect* ins, StepState* st, const Frame& F, c
 
 }  // namespace
 
-// The FP64 frame block (one thread): body and wing orientations and angular
-// velocities, pivots, and the parts' bounding boxes.  frac = 0: at the state's
-// time; frac > 0: at t0 + frac dt of the current step (the later RK4 stages,
-// after k_scalars has written t0 and dt).
-static __device__ void kinematics_frame(const flusi_insect* ins, const StepState* st, const StepCoef* coef,
-                                        Frame* fr, double h, double frac, const Member* mb)
+// ---- the frame block, by one warp.
+//
+// FP64 instructions cost the same with one lane active as with 32, and each
+// waits for the one before it: on one thread the frame block was a chain of
+// some two thousand of them (48 to 100 us a step, the longest kernel of a small
+// grid).  Here every level of the computation is spread over lanes and handed
+// on through shared memory: a harmonic per lane, an angle's sine and cosine per
+// lane, an element of a matrix product per lane, a component of a rotated
+// vector per lane, a corner of a bounding box per lane: 18 to 23 us.  A step of
+// 48 x 36 x 24 went from 105 to 63 us with it; RK4 at 192^3, with contour wings
+// and the later stages' frames beside the passes, from 1335 to 1044 us.
+struct KinWork {
+    flusi_insect I;
+    Frame F;
+    double harm[3][FLUSI_MAX_FOURIER][3];   // per angle and harmonic: value, first and second derivative
+    double ang[3][3];                       // phi, alpha, theta and their derivatives
+    double cs[8], sn[8];                    // psi, beta, gamma, eta_stroke, alpha, theta, phi, pi
+    double Bx[9], By[9], Bz[9], B1[9];      // body rotations
+    double Rt[9], Rpi[9], Ra[2][9], Rp[2][9], Ms[2][9], T[2][9], Mw[2][9];
+    double vec[3][3];                       // angular velocities on their way to the global frame
+    double rp[2][3], drp[2][3], in[2][3], din[2][3], v[2][3], dv[2][3];
+    double lo[3], hi[3], rim, corner[3][8][3], arc[8][2];
+};
+
+// element e = 3 r + c of the rotation about an axis (rot_x, rot_y, rot_z)
+__device__ double rot_elem(int axis, double c, double s, int e)
 {
+    const int r = e / 3, k = e - 3 * r;
+    if (r == axis || k == axis) return r == k ? 1.0 : 0.0;
+    if (r == k) return c;
+    // the next axis in cyclic order carries +s
+    return k == (r + 1) % 3 ? s : -s;
+}
+// element of A B, of A^T x and of A x
+__device__ double mul_elem(const double* A, const double* B, int e)
+{
+    const int i = e / 3, j = e - 3 * i;
+    return A[i * 3] * B[j] + A[i * 3 + 1] * B[3 + j] + A[i * 3 + 2] * B[6 + j];
+}
+__device__ double apply_t_elem(const double* A, const double* x, int i)
+{
+    return A[i] * x[0] + A[3 + i] * x[1] + A[6 + i] * x[2];
+}
+__device__ double apply_elem(const double* A, const double* x, int i)
+{
+    return A[3 * i] * x[0] + A[3 * i + 1] * x[1] + A[3 * i + 2] * x[2];
+}
+__device__ double cross_elem(const double* a, const double* b, int i)
+{
+    const int j = (i + 1) % 3, k = (i + 2) % 3;
+    return a[j] * b[k] - a[k] * b[j];
+}
+
+// Body and wing orientations and angular velocities, pivots, and the parts'
+// bounding boxes at time t, into w.F; h grows the boxes.  All 32 lanes call it.
+__device__ void kinematics_frame(KinWork& w, double t, double h, int lane)
+{
+    const flusi_insect& I = w.I;
+    Frame& F = w.F;
+    const int trio = lane / 3, comp = lane - 3 * trio;     // lanes as triples of components
+    const int nine = lane / 9, elem = lane - 9 * nine;     // lanes as matrices
+    const bool flying = I.free_flight != 0;
+
+    // ---- the angles' Fourier series and derivatives
+    if (lane < 3 * FLUSI_MAX_FOURIER) {
+        const int a = lane / FLUSI_MAX_FOURIER, i = lane - a * FLUSI_MAX_FOURIER;
+        if (i < I.nfourier) {
+            const double ca = a == 0 ? I.phi_a[i] : a == 1 ? I.alpha_a[i] : I.theta_a[i];
+            const double cb = a == 0 ? I.phi_b[i] : a == 1 ? I.alpha_b[i] : I.theta_b[i];
+            const double two_pi = 6.283185307179586476925286766559;
+            const double om = two_pi * (i + 1) * I.freq;
+            double sn, cs;
+            sincos(om * t, &sn, &cs);
+            const double c = ca * cs + cb * sn;
+            w.harm[a][i][0] = c;
+            w.harm[a][i][1] = om * (cb * cs - ca * sn);
+            w.harm[a][i][2] = -(om * om * c);
+        }
+    }
+    if (lane < 3) {
+        F.xc[lane] = I.x_cntr[lane];
+        F.uc[lane] = I.u_cntr[lane];
+    }
+    if (lane == 31) F.t = t;
+    __syncwarp();
+    if (lane < 9) {
+        double acc = comp == 0 ? 0.5 * (trio == 0 ? I.phi_a0 : trio == 1 ? I.alpha_a0 : I.theta_a0) : 0.0;
+        for (int i = 0; i < I.nfourier; ++i) acc += w.harm[trio][i][comp];
+        w.ang[trio][comp] = acc;
+    }
+    __syncwarp();
+    const double dphi = w.ang[0][1], dalpha = w.ang[1][1], dtheta = w.ang[2][1];
+
+    // ---- sines and cosines, then the elementary rotations
+    if (lane < 8) {
+        const double pi = 3.141592653589793238462643383279;
+        const double x = lane == 0 ? I.psi : lane == 1 ? I.beta : lane == 2 ? I.gamma : lane == 3 ? I.eta_stroke
+                         : lane == 4 ? w.ang[1][0] : lane == 5 ? w.ang[2][0] : lane == 6 ? w.ang[0][0] : pi;
+        sincos(x, &w.sn[lane], &w.cs[lane]);
+    }
+    __syncwarp();
+    // the right wing mirrors the left: R_x(pi) in the stroke matrix and
+    // (phi, alpha) -> (-phi, -alpha) in the wing matrix
+    if (nine == 0) {
+        w.Bx[elem] = rot_elem(0, w.cs[0], w.sn[0], elem);
+        w.Ms[0][elem] = rot_elem(1, w.cs[3], w.sn[3], elem);
+        w.Ra[0][elem] = rot_elem(1, w.cs[4], w.sn[4], elem);
+        w.Rp[0][elem] = rot_elem(0, w.cs[6], w.sn[6], elem);
+    } else if (nine == 1) {
+        w.By[elem] = rot_elem(1, w.cs[1], w.sn[1], elem);
+        w.Rpi[elem] = rot_elem(0, w.cs[7], w.sn[7], elem);
+        w.Ra[1][elem] = rot_elem(1, w.cs[4], -w.sn[4], elem);
+        w.Rp[1][elem] = rot_elem(0, w.cs[6], -w.sn[6], elem);
+    } else if (nine == 2) {
+        w.Bz[elem] = rot_elem(2, w.cs[2], w.sn[2], elem);
+        w.Rt[elem] = rot_elem(2, w.cs[5], -w.sn[5], elem);
+    }
+    __syncwarp();
+    // M_body = R_x R_y R_z (Sec. 3.1), or the quaternion's (Sec. 3.6)
+    if (nine < 2) w.T[nine][elem] = mul_elem(w.Ra[nine], w.Rt, elem);
+    else if (nine == 2) w.B1[elem] = mul_elem(w.Bx, w.By, elem);
+    __syncwarp();
+    if (nine < 2) {
+        w.Mw[nine][elem] = mul_elem(w.T[nine], w.Rp[nine], elem);
+    } else if (nine == 2) {
+        double m = mul_elem(w.B1, w.Bz, elem);
+        if (flying) {
+            const M3 Q = quat_to_global(I.quat);
+            const int at = 3 * (elem % 3) + elem / 3;   // its transpose
+            for (int i = 0; i < 9; ++i)
+                if (i == at) m = Q.a[i];
+        }
+        F.Mb[elem] = m;
+    }
+    if (nine == 0) w.Ms[1][elem] = mul_elem(w.Rpi, w.Ms[0], elem);
+    __syncwarp();
+    if (nine < 2) w.T[nine][elem] = mul_elem(w.Mw[nine], w.Ms[nine], elem);
+    __syncwarp();
+    if (nine < 2) F.Mw[nine][elem] = mul_elem(w.T[nine], F.Mb, elem);   // global -> wing frame
+
+    // ---- angular velocities: triples 0, 1 the wings (stroke frame, then body,
+    // then global), triple 2 the body (nested form of Sec. 3.1)
+    if (lane < 9)
+        w.vec[trio][comp] = trio < 2 ? (comp == 1 ? (trio == 0 ? dalpha : -dalpha) : 0.0) : (comp == 0 ? I.psi_dot : 0.0);
+    __syncwarp();
+    for (int k = 0; k < 5; ++k) {
+        double y = 0.0;
+        const bool on = lane < 9 && (trio < 2 || k < 3);
+        if (on) {
+            const double* A = trio == 2 ? (k == 0 ? w.Bx : k == 1 ? w.By : w.Bz)
+                                        : (k == 0 ? w.Ra[trio] : k == 1 ? w.Rt : k == 2 ? w.Rp[trio] : k == 3 ? w.Ms[trio] : F.Mb);
+            y = apply_t_elem(A, w.vec[trio], comp);
+            if (trio < 2 && k == 0 && comp == 2) y += -dtheta;
+            if (trio < 2 && k == 1 && comp == 0) y += trio == 0 ? dphi : -dphi;
+            if (trio == 2 && k == 0 && comp == 1) y += I.beta_dot;
+            if (trio == 2 && k == 1 && comp == 2) y += I.gamma_dot;
+        }
+        __syncwarp();
+        if (on) w.vec[trio][comp] = y;
+        __syncwarp();
+    }
+    if (lane < 6) F.Ow[trio][comp] = w.vec[trio][comp];
+    else if (lane < 9) F.Ob[comp] = flying ? apply_t_elem(F.Mb, I.Omega_body, comp) : w.vec[2][comp];
+
+    // In the wing frame Omega^(w) = e_a + Ra (e_t + Rt e_p) with
+    // e_a = (0, alpha', 0), e_t = (0, 0, -theta'), e_p = (phi', 0, 0).  Both
+    // factors are rotations about one fixed axis, so d/dt (Ra x) =
+    // Ra x' - e_a x (Ra x) and d/dt (Rt x) = Rt x' - e_t x (Rt x).
+    {
+        const double sg = trio == 0 ? 1.0 : -1.0;
+        const double ea[3] = {0, sg * dalpha, 0}, et[3] = {0, 0, -dtheta}, ep[3] = {sg * dphi, 0, 0};
+        const double dea[3] = {0, sg * w.ang[1][2], 0}, det[3] = {0, 0, -w.ang[2][2]};
+        const double dep[3] = {sg * w.ang[0][2], 0, 0};
+        if (lane < 6) {
+            w.rp[trio][comp] = apply_elem(w.Rt, ep, comp);
+            w.drp[trio][comp] = apply_elem(w.Rt, dep, comp);
+        }
+        __syncwarp();
+        if (lane < 6) {
+            w.in[trio][comp] = (comp == 2 ? et[2] : 0.0) + w.rp[trio][comp];
+            w.din[trio][comp] = (comp == 2 ? det[2] : 0.0) + w.drp[trio][comp] - cross_elem(et, w.rp[trio], comp);
+        }
+        __syncwarp();
+        if (lane < 6) {
+            w.v[trio][comp] = apply_elem(w.Ra[trio], w.in[trio], comp);
+            w.dv[trio][comp] = apply_elem(w.Ra[trio], w.din[trio], comp);
+        }
+        __syncwarp();
+        if (lane < 6) {
+            F.Oww[trio][comp] = (comp == 1 ? ea[1] : 0.0) + w.v[trio][comp];
+            F.dOww[trio][comp] = (comp == 1 ? dea[1] : 0.0) + w.dv[trio][comp] - cross_elem(ea, w.v[trio], comp);
+            const double* pb = trio == 0 ? I.pivot_l : I.pivot_r;
+            F.pv[trio][comp] = F.xc[comp] + apply_t_elem(F.Mb, pb, comp);
+        }
+    }
+
+    // ---- bounding boxes (global) of the region where chi > 0
+    // body-frame box of thorax, head and eyes; its corners, grown by h
+    if (I.body_type == 3 && lane < 8) {
+        // the arc x = x_c + r_c sin th, z = z_c + r_c cos th over
+        // th0 -+ a/r_c: its ends and the quarter angles inside, grown by b
+        const double rc = I.body_arc[0], xc = I.body_arc[1], zc = I.body_arc[2];
+        const double th0 = atan2(-xc, -zc), t1 = th0 - I.body_a / rc, t2 = th0 + I.body_a / rc;
+        const double half_pi = 1.5707963267948966192313216916398;
+        const int k1 = (int)ceil(t1 / half_pi), k2 = (int)floor(t2 / half_pi);
+        const int k = min(k1 - 1 + lane, k2 + 1);   // at most 4 quarter angles in an arc under a full turn
+        const double th = k < k1 ? t1 : k > k2 ? t2 : k * half_pi;
+        w.arc[lane][0] = xc + rc * sin(th);
+        w.arc[lane][1] = zc + rc * cos(th);
+    }
+    double rim = 0.0;   // R(theta) <= a0/2 + sum sqrt(a_i^2 + b_i^2)
+    if (I.wing_shape == 1) {
+        if (lane < I.ncontour)
+            rim = sqrt(I.contour_a[lane] * I.contour_a[lane] + I.contour_b[lane] * I.contour_b[lane]);
+        for (int o = 16; o > 0; o >>= 1) rim += __shfl_xor_sync(0xffffffffu, rim, o);
+        rim += 0.5 * I.contour_a0;
+    }
+    __syncwarp();
+    if (lane < 3) {
+        const double ey = I.body_type == 1 ? I.body_a : I.body_b;
+        double lo = lane == 0 ? -I.body_a : -ey, hi = lane == 0 ? I.body_a : ey;
+        if (I.body_type == 3 && lane != 1) {
+            lo = 1e300;
+            hi = -1e300;
+            for (int k = 0; k < 8; ++k) {
+                const double p = w.arc[k][lane == 0 ? 0 : 1];
+                lo = fmin(lo, p - I.body_b);
+                hi = fmax(hi, p + I.body_b);
+            }
+        }
+        if (I.body_type >= 2 && I.head_r > 0) {
+            lo = fmin(lo, I.head_x0[lane] - I.head_r);
+            hi = fmax(hi, I.head_x0[lane] + I.head_r);
+        }
+        if (I.body_type >= 2 && I.eye_r > 0) {
+            const double c = I.eye_x0[lane], m = lane == 1 ? -c : c;   // both eyes
+            lo = fmin(lo, fmin(c, m) - I.eye_r);
+            hi = fmax(hi, fmax(c, m) + I.eye_r);
+        }
+        w.lo[lane] = lo;
+        w.hi[lane] = hi;
+    }
+    __syncwarp();
+    if (lane < 24) {
+        const int part = lane / 8, c = lane - 8 * part;
+        double q[3];
+        if (part == 0) {
+            for (int i = 0; i < 3; ++i) q[i] = (c >> i) & 1 ? w.hi[i] + h : w.lo[i] - h;
+        } else if (I.wing_shape == 1) {
+            q[0] = c & 1 ? I.contour_xc + rim + h : I.contour_xc - rim - h;
+            q[1] = c & 2 ? I.contour_yc + rim + h : I.contour_yc - rim - h;
+            q[2] = c & 4 ? 0.5 * I.wing_h + h : -0.5 * I.wing_h - h;
+        } else {
+            q[0] = c & 1 ? I.wing_c_le + h : -I.wing_c_te - h;
+            q[1] = c & 2 ? I.wing_R + h : -h;
+            q[2] = c & 4 ? 0.5 * I.wing_h + h : -0.5 * I.wing_h - h;
+        }
+        const double* M = part == 0 ? F.Mb : F.Mw[part - 1];
+        const double* at = part == 0 ? F.xc : F.pv[part - 1];
+        for (int i = 0; i < 3; ++i) w.corner[part][c][i] = at[i] + apply_t_elem(M, q, i);
+    }
+    __syncwarp();
+    if (lane < 18) {
+        const int part = lane / 6, b = lane - 6 * part;
+        const bool present = part == 0 ? I.body_type != 0 : part <= I.nwings;
+        double v = b & 1 ? -1e300 : 1e300;
+        if (present)
+            for (int c = 0; c < 8; ++c) v = b & 1 ? fmax(v, w.corner[part][c][b / 2]) : fmin(v, w.corner[part][c][b / 2]);
+        F.box[part][b] = v;
+        if (b == 0) F.active[part] = present ? 1 : 0;
+    } else if (lane == 18) {
+        F.pad = 0;
+    }
+    __syncwarp();
+}
+
+// One warp: the FP64 frame block at the state's time (frac = 0) or at
+// t0 + frac dt of the current step (the later RK4 stages, after k_scalars has
+// written t0 and dt) and, with `with_t`, its FP32 and FP64 copies with the
+// mask shape S (FrameT, at their offsets of the frame slot) for the x pass.
+__global__ void __launch_bounds__(32)
+k_kinematics(const flusi_insect* ins, const StepState* st, const StepCoef* coef, Frame* fr, double h, double frac,
+             const Member* mb, const __grid_constant__ Shape S, int with_t, double inv_eta)
+{
+    __shared__ KinWork w;
     if (mb) {
         const Member& m = mb[blockIdx.z];
         ins = m.ins;
@@ -185,189 +402,19 @@ static __device__ void kinematics_frame(const flusi_insect* ins, const StepState
         coef = m.coef;
         fr = m.fr;
     }
-    const double t = frac > 0.0 ? coef->t0 + frac * coef->dt : st->t;
-    Frame F;
-    F.t = t;
-    for (int i = 0; i < 3; ++i) {
-        F.xc[i] = ins->x_cntr[i];
-        F.uc[i] = ins->u_cntr[i];
-    }
-    M3 Mb;
-    if (ins->free_flight) {
-        // Sec. 3.6: the orientation is the quaternion's, Omega^(b) is state
-        const M3 Q = quat_to_global(ins->quat);
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) Mb.a[3 * i + j] = Q.a[3 * j + i];
-        apply(Q, ins->Omega_body, F.Ob);
-    } else {
-        // body frame: yaw, then pitch, then roll
-        M3 Rx = rot_x(ins->psi), Ry = rot_y(ins->beta), Rz = rot_z(ins->gamma);
-        Mb = mul(mul(Rx, Ry), Rz);
-        // body angular velocity in the global frame (nested form of Sec. 3.1)
-        double v[3] = {ins->psi_dot, 0, 0};
-        apply_t(Rx, v, v);
-        v[1] += ins->beta_dot;
-        apply_t(Ry, v, v);
-        v[2] += ins->gamma_dot;
-        apply_t(Rz, v, F.Ob);
-    }
-    for (int i = 0; i < 9; ++i) F.Mb[i] = Mb.a[i];
-
-    double phi, alpha, theta, dphi, dalpha, dtheta, ddphi, ddalpha, ddtheta;
-    int nf = ins->nfourier;
-    series(ins->phi_a0, ins->phi_a, ins->phi_b, nf, ins->freq, t, &phi, &dphi, &ddphi);
-    series(ins->alpha_a0, ins->alpha_a, ins->alpha_b, nf, ins->freq, t, &alpha, &dalpha, &ddalpha);
-    series(ins->theta_a0, ins->theta_a, ins->theta_b, nf, ins->freq, t, &theta, &dtheta, &ddtheta);
-
-    const double pi = 3.141592653589793238462643383279;
-    for (int s = 0; s < 2; ++s) {
-        // the right wing mirrors the left: R_x(pi) in the stroke matrix and
-        // (phi, alpha) -> (-phi, -alpha) in the wing matrix
-        double sg = s == 0 ? 1.0 : -1.0;
-        M3 Ms = rot_y(ins->eta_stroke);
-        if (s == 1) Ms = mul(rot_x(pi), Ms);
-        M3 Ra = rot_y(sg * alpha), Rt = rot_z(-theta), Rp = rot_x(sg * phi);
-        M3 Mw = mul(mul(Ra, Rt), Rp);
-        M3 Mg = mul(mul(Mw, Ms), Mb);          // global -> wing frame
-        for (int i = 0; i < 9; ++i) F.Mw[s][i] = Mg.a[i];
-        // angular velocity in the stroke frame, then body, then global frame
-        double w[3] = {0, sg * dalpha, 0};
-        apply_t(Ra, w, w);
-        w[2] += -dtheta;
-        apply_t(Rt, w, w);
-        w[0] += sg * dphi;
-        apply_t(Rp, w, w);
-        apply_t(Ms, w, w);
-        apply_t(Mb, w, F.Ow[s]);
-        // In the wing frame Omega^(w) = e_a + Ra (e_t + Rt e_p) with
-        // e_a = (0, alpha', 0), e_t = (0, 0, -theta'), e_p = (phi', 0, 0).  Both
-        // factors are rotations about one fixed axis, so d/dt (Ra x) =
-        // Ra x' - e_a x (Ra x) and d/dt (Rt x) = Rt x' - e_t x (Rt x).
-        {
-            const double ea[3] = {0, sg * dalpha, 0}, et[3] = {0, 0, -dtheta}, ep[3] = {sg * dphi, 0, 0};
-            const double dea[3] = {0, sg * ddalpha, 0}, det[3] = {0, 0, -ddtheta};
-            const double dep[3] = {sg * ddphi, 0, 0};
-            double rp[3], in[3], v[3], dv[3], c[3], drp[3];
-            apply(Rt, ep, rp);                          // Rt e_p
-            for (int i = 0; i < 3; ++i) in[i] = et[i] + rp[i];
-            apply(Ra, in, v);                           // Ra (e_t + Rt e_p)
-            for (int i = 0; i < 3; ++i) F.Oww[s][i] = ea[i] + v[i];
-            apply(Rt, dep, drp);
-            cross3(et, rp, c);
-            for (int i = 0; i < 3; ++i) dv[i] = det[i] + drp[i] - c[i];
-            apply(Ra, dv, dv);
-            cross3(ea, v, c);
-            for (int i = 0; i < 3; ++i) F.dOww[s][i] = dea[i] + dv[i] - c[i];
-        }
-        const double* pb = s == 0 ? ins->pivot_l : ins->pivot_r;
-        double pg[3];
-        apply_t(Mb, pb, pg);
-        for (int i = 0; i < 3; ++i) F.pv[s][i] = F.xc[i] + pg[i];
-    }
-
-    // bounding boxes (global) of the region where chi > 0
-    for (int p = 0; p < 3; ++p) {
-        for (int i = 0; i < 3; ++i) {
-            F.box[p][2 * i] = 1e300;
-            F.box[p][2 * i + 1] = -1e300;
-        }
-        F.active[p] = 0;
-    }
-    if (ins->body_type != 0) {
-        // body-frame box of thorax, head and eyes, grown by h; its corners in
-        // the global frame
-        double lo[3], hi[3];
-        const double ey = ins->body_type == 1 ? ins->body_a : ins->body_b;
-        lo[0] = -ins->body_a;
-        hi[0] = ins->body_a;
-        lo[1] = lo[2] = -ey;
-        hi[1] = hi[2] = ey;
-        if (ins->body_type == 3) {
-            // the arc x = x_c + r_c sin th, z = z_c + r_c cos th over
-            // th0 -+ a/r_c: its ends and the quarter angles inside, grown by b
-            const double rc = ins->body_arc[0], xc = ins->body_arc[1], zc = ins->body_arc[2];
-            const double th0 = atan2(-xc, -zc), t1 = th0 - ins->body_a / rc, t2 = th0 + ins->body_a / rc;
-            const double half_pi = 1.5707963267948966192313216916398;
-            lo[0] = lo[2] = 1e300;
-            hi[0] = hi[2] = -1e300;
-            const int k1 = (int)ceil(t1 / half_pi), k2 = (int)floor(t2 / half_pi);
-            for (int k = k1 - 1; k <= k2 + 1; ++k) {
-                const double th = k < k1 ? t1 : k > k2 ? t2 : k * half_pi;
-                const double px = xc + rc * sin(th), pz = zc + rc * cos(th);
-                lo[0] = fmin(lo[0], px - ins->body_b);
-                hi[0] = fmax(hi[0], px + ins->body_b);
-                lo[2] = fmin(lo[2], pz - ins->body_b);
-                hi[2] = fmax(hi[2], pz + ins->body_b);
-            }
-        }
-        if (ins->body_type >= 2 && ins->head_r > 0)
-            for (int i = 0; i < 3; ++i) {
-                lo[i] = fmin(lo[i], ins->head_x0[i] - ins->head_r);
-                hi[i] = fmax(hi[i], ins->head_x0[i] + ins->head_r);
-            }
-        if (ins->body_type >= 2 && ins->eye_r > 0)
-            for (int i = 0; i < 3; ++i) {
-                const double c = ins->eye_x0[i], m = i == 1 ? -c : c;   // both eyes
-                lo[i] = fmin(lo[i], fmin(c, m) - ins->eye_r);
-                hi[i] = fmax(hi[i], fmax(c, m) + ins->eye_r);
-            }
-        for (int c = 0; c < 8; ++c) {
-            double q[3] = {(c & 1 ? hi[0] : lo[0]) + (c & 1 ? h : -h),
-                           (c & 2 ? hi[1] : lo[1]) + (c & 2 ? h : -h),
-                           (c & 4 ? hi[2] : lo[2]) + (c & 4 ? h : -h)}, gq[3];
-            apply_t(Mb, q, gq);
-            for (int i = 0; i < 3; ++i) gq[i] += F.xc[i];
-            box_grow(F.box[0], gq);
-        }
-        F.active[0] = 1;
-    }
-    for (int s = 0; s < ins->nwings && s < 2; ++s) {
-        M3 Mg;
-        for (int i = 0; i < 9; ++i) Mg.a[i] = F.Mw[s][i];
-        double xs[2] = {-ins->wing_c_te - h, ins->wing_c_le + h};
-        double ys[2] = {-h, ins->wing_R + h};
-        double zs[2] = {-0.5 * ins->wing_h - h, 0.5 * ins->wing_h + h};
-        if (ins->wing_shape == 1) {
-            // R(theta) <= a0/2 + sum sqrt(a_i^2 + b_i^2)
-            double rb = 0.5 * ins->contour_a0;
-            for (int i = 0; i < ins->ncontour; ++i)
-                rb += sqrt(ins->contour_a[i] * ins->contour_a[i] + ins->contour_b[i] * ins->contour_b[i]);
-            xs[0] = ins->contour_xc - rb - h;
-            xs[1] = ins->contour_xc + rb + h;
-            ys[0] = ins->contour_yc - rb - h;
-            ys[1] = ins->contour_yc + rb + h;
-        }
-        for (int c = 0; c < 8; ++c) {
-            double q[3] = {xs[c & 1], ys[(c >> 1) & 1], zs[(c >> 2) & 1]}, g[3];
-            apply_t(Mg, q, g);
-            for (int i = 0; i < 3; ++i) g[i] += F.pv[s][i];
-            box_grow(F.box[1 + s], g);
-        }
-        F.active[1 + s] = 1;
-    }
-    *fr = F;
-}
-
-// One warp.  Thread 0 forms the FP64 frame block; with `with_t`, the warp
-// then writes its FP32 and FP64 copies with the mask shape S (FrameT, at their
-// offsets of the frame slot) for the x pass.
-__global__ void k_kinematics(const flusi_insect* ins, const StepState* st, const StepCoef* coef, Frame* fr,
-                             double h, double frac, const Member* mb, Shape S, int with_t, double inv_eta)
-{
-    __shared__ Shape sS;
-    if (blockIdx.x != 0) return;
-    if (mb) fr = mb[blockIdx.z].fr;
-    if (threadIdx.x == 0) {
-        kinematics_frame(ins, st, coef, fr, h, frac, mb);
-        if (with_t) sS = S;
-    }
-    if (!with_t || threadIdx.x >= 32) return;
-    __syncwarp();
     const int lane = threadIdx.x;
-    frame_to_t<float>(const_cast<FrameT<float>*>(frame_t<float>(fr)), fr, &sS, inv_eta, lane);
-    frame_to_t<double>(const_cast<FrameT<double>*>(frame_t<double>(fr)), fr, &sS, inv_eta, lane);
+    static_assert(sizeof(flusi_insect) % 8 == 0 && sizeof(Frame) % 8 == 0, "word copies");
+    for (int i = lane; i < (int)(sizeof(flusi_insect) / 8); i += 32)
+        reinterpret_cast<double*>(&w.I)[i] = reinterpret_cast<const double*>(ins)[i];
+    const double t = frac > 0.0 ? coef->t0 + frac * coef->dt : st->t;
+    __syncwarp();
+    kinematics_frame(w, t, h, lane);
+    for (int i = lane; i < (int)(sizeof(Frame) / 8); i += 32)
+        reinterpret_cast<double*>(fr)[i] = reinterpret_cast<const double*>(&w.F)[i];
+    if (!with_t) return;
+    frame_to_t<float>(const_cast<FrameT<float>*>(frame_t<float>(fr)), &w.F, &S, inv_eta, lane);
+    frame_to_t<double>(const_cast<FrameT<double>*>(frame_t<double>(fr)), &w.F, &S, inv_eta, lane);
 }
-
 
 // A bounded wait on a barrier that nothing completes (the arrival count is 2
 // and one thread arrives once): gives up after max_cycles and reports as the
