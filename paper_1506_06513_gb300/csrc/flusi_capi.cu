@@ -422,7 +422,7 @@ cudaError_t enqueue_step(flusi_t h, cudaStream_t s, cudaEvent_t* ev, const char*
         if (q == 0) {
             mark("scalars");
             double3 opts = make_double3(h->opt.cfl, h->opt.dt_fixed, h->opt.dt_max);
-            k_scalars<<<dim3(1, 1, current_batch().n), 256, 0, sk>>>(g, at<double>(h, h->opart), h->xgrid, st, coef, at<double>(h, h->orows),
+            k_scalars<<<dim3(kScalarCtas, 1, current_batch().n), 256, 0, sk>>>(g, at<double>(h, h->opart), h->xgrid, st, coef, at<double>(h, h->orows),
                                          h->opt.force_ring, at<double>(h, h->oetab), opts, rk4_dt_diff(h),
                                          at<Frame>(h, h->oframe), at<flusi_insect>(h, h->oins), current_batch().mb);
             if ((e = cudaGetLastError())) return e;
@@ -674,7 +674,12 @@ int flusi_bind(flusi_t h, void* ws, size_t bytes, void* stream)
         CK(cudaMemcpyAsync(h->ws + h->oins, &h->ins, sizeof h->ins, cudaMemcpyHostToDevice, h->stream), "insect");
     CK(cudaStreamSynchronize(h->stream), "bind");
     if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking), "capture stream");
-    if (!h->side) CK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking), "side stream");
+    if (!h->side) {
+        // the small kernels go first where they compete with a pass for an SM
+        int low = 0, high = 0;
+        CK(cudaDeviceGetStreamPriorityRange(&low, &high), "stream priorities");
+        CK(cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, high), "side stream");
+    }
     for (cudaEvent_t* ev : {&h->ev_fork, &h->ev_kin, &h->ev_x, &h->ev_sc})
         if (!*ev) CK(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "step events");
     h->bound = 1;

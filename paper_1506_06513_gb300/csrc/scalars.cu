@@ -6,6 +6,8 @@
 //    AB2 coefficients and exponential tables, and the force row
 //    (Eqs. force_with_unst_corrections, moment_of_love);
 //  * reset: the step state after a new initial condition.
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 #include "../../include/flusi.h"
@@ -440,21 +442,30 @@ __global__ void k_reset_state(StepState* st, StepCoef* coef)
     *coef = c;
 }
 
-// One block.  Reduces part[nparts][kNumSums] in a fixed order, then forms the
-// step's scalars.  `opts` = {cfl, dt_fixed, dt_max}; dt_diff > 0 caps the
-// adaptive step (the explicit-diffusion limit of RK4).
+// A cluster of CTAs per solver.  Reduces part[nparts][kNumSums] in a fixed
+// order, then forms the step's scalars.  `opts` = {cfl, dt_fixed, dt_max};
+// dt_diff > 0 caps the adaptive step (the explicit-diffusion limit of RK4).
 //
 // FP64 arithmetic is a small fraction of FP32 here, and a warp instruction
 // costs the FP64 units the same with one lane active as with 32: the work is
-// spread over lanes (a slot and segment of CTAs per thread, a force or moment
-// component per lane) and each scalar is computed once, not by every thread.
-constexpr int kScalarSeg = 6;   // CTA segments per slot: kNumSums * 6 = 240 threads
+// spread over lanes (a slot and segment of the physical pass's CTAs per thread,
+// a force or moment component per lane), and over the FP64 units of several
+// SMs: every CTA of the cluster sums its share of the partials, takes the
+// others' sums through distributed shared memory in rank order (so all hold the
+// same totals and dt) and fills its share of the factor tables, rank 0 the force
+// row meanwhile.  On one block it took 16 to 61 us, longer than the forward
+// passes beside it wherever the physical pass has many small tiles.
+constexpr int kScalarSeg = 6;   // segments of a CTA's share per slot: kNumSums * 6 = 240 threads
 static_assert(kNumSums * kScalarSeg <= 256, "k_scalars runs 256 threads");
 
-__global__ void k_scalars(Geom g, const double* part, int nparts, StepState* st, StepCoef* coef, double* rows,
-                          int ring, double* etab, double3 opts, double dt_diff, const Frame* fr, flusi_insect* ins,
-                          const Member* mb)
+__global__ void __cluster_dims__(kScalarCtas, 1, 1) __launch_bounds__(256)
+k_scalars(Geom g, const double* part, int nparts, StepState* st, StepCoef* coef, double* rows,
+          int ring, double* etab, double3 opts, double dt_diff, const Frame* fr, flusi_insect* ins,
+          const Member* mb)
 {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
     if (mb) {
         const Member& m = mb[blockIdx.z];
         part = m.part;
@@ -467,48 +478,60 @@ __global__ void k_scalars(Geom g, const double* part, int nparts, StepState* st,
         g.nu = m.nu;
     }
     __shared__ double seg[kNumSums][kScalarSeg];
+    __shared__ double own[kNumSums];
     __shared__ double tot[kNumSums];
     __shared__ double sh_dt;
     const int tid = threadIdx.x, T = blockDim.x;
 
-    // every thread reads the state before the first barrier; thread 0 writes
-    // it only after the last one
+    // every thread of the cluster reads the state before the first cluster
+    // barrier; rank 0's thread 0 writes it only after that
     const int status = st->status;
     const long long n = st->n;
     const double dt_prev = st->dt_prev;
     if (status != 0) {
-        if (tid == 0) coef->skip = 1;
-        return;
+        if (rank == 0 && tid == 0) coef->skip = 1;
+        return;   // the whole cluster
     }
-    // slot k, segment s: the partials of CTAs [s c, (s + 1) c) in order; then
-    // the segments in order
+    // slot k, segment s of this CTA: the partials of CTAs [s c, (s + 1) c) in
+    // order; then the segments in order
     if (tid < kNumSums * kScalarSeg) {
-        const int k = tid % kNumSums, sg = tid / kNumSums;
-        const int chunk = (nparts + kScalarSeg - 1) / kScalarSeg;
+        const int k = tid % kNumSums, sg = rank * kScalarSeg + tid / kNumSums;
+        const int chunk = (nparts + kScalarCtas * kScalarSeg - 1) / (kScalarCtas * kScalarSeg);
         const int i0 = sg * chunk, i1 = min(nparts, i0 + chunk);
         const bool is_max = (k == kSumUmax2 || k == kSumBad);
         double acc = 0.0;
-#pragma unroll 4
+#pragma unroll 8
         for (int i = i0; i < i1; ++i) {
             const double v = part[(size_t)i * kNumSums + k];
             acc = is_max ? fmax(acc, v) : acc + v;
         }
-        seg[k][sg] = acc;
+        seg[k][tid / kNumSums] = acc;
     }
     __syncthreads();
     if (tid < kNumSums) {
         const bool is_max = (tid == kSumUmax2 || tid == kSumBad);
         double a = 0.0;
         for (int s2 = 0; s2 < kScalarSeg; ++s2) a = is_max ? fmax(a, seg[tid][s2]) : a + seg[tid][s2];
+        own[tid] = a;
+    }
+    cluster.sync();
+    if (tid < kNumSums) {
+        const bool is_max = (tid == kSumUmax2 || tid == kSumBad);
+        double a = 0.0;
+        for (int r = 0; r < kScalarCtas; ++r) {
+            const double v = cluster.map_shared_rank(own, r)[tid];
+            a = is_max ? fmax(a, v) : a + v;
+        }
         tot[tid] = a;
     }
     __syncthreads();
 
     if (tot[kSumBad] != 0.0) {
-        if (tid == 0) {
+        if (rank == 0 && tid == 0) {
             st->status = FLUSI_ENONFINITE;
             coef->skip = 1;
         }
+        cluster.sync();   // the others have read this CTA's sums
         return;
     }
 
@@ -538,7 +561,7 @@ __global__ void k_scalars(Geom g, const double* part, int nparts, StepState* st,
     const double two_pi = 6.283185307179586476925286766559;
     const int Mt = g.Mx + g.My + g.Mz;
     float* etab32 = reinterpret_cast<float*>(etab + 2 * Mt);
-    for (int i = tid; i < 2 * Mt; i += T) {
+    for (int i = (rank - 1) * T + tid; rank > 0 && i < 2 * Mt; i += (kScalarCtas - 1) * T) {
         int which = i / Mt, r = i % Mt;
         double k, tau = which == 0 ? dt : dt + dt_prev;
         if (r < g.Mx) k = two_pi * r / g.Lx;
@@ -549,73 +572,76 @@ __global__ void k_scalars(Geom g, const double* part, int nparts, StepState* st,
         etab32[i] = float(e);
     }
 
-    // force row: lane 3 p + i of warp 0 takes component i of part p; then the
-    // wing power (lanes 0, 1) and the rest (lane 0)
-    double* row = rows + (size_t)(n % ring) * kRowCols;
-    if (tid < 9) {
-        const int p = tid / 3, i = tid % 3;
-        const double dV = g.dx * g.dy * g.dz;
-        const double* s = tot + 12 * p;
-        double Fv = s[i] * dV / g.eta, Mv = s[3 + i] * dV / g.eta;
-        const double Is = s[6 + i] * dV, Js = s[9 + i] * dV;
-        if (!first) {
-            const double inv_dtp = 1.0 / dt_prev;
-            Fv += (Is - st->Is_prev[p][i]) * inv_dtp;
-            Mv += (Js - st->Js_prev[p][i]) * inv_dtp;
+    // force row: lane 3 p + i of rank 0's warp 0 takes component i of part p;
+    // then the wing power (lanes 0, 1) and the rest (lane 0)
+    if (rank == 0 && tid < 32) {
+        double* row = rows + (size_t)(n % ring) * kRowCols;
+        if (tid < 9) {
+            const int p = tid / 3, i = tid % 3;
+            const double dV = g.dx * g.dy * g.dz;
+            const double* s = tot + 12 * p;
+            double Fv = s[i] * dV / g.eta, Mv = s[3 + i] * dV / g.eta;
+            const double Is = s[6 + i] * dV, Js = s[9 + i] * dV;
+            if (!first) {
+                const double inv_dtp = 1.0 / dt_prev;
+                Fv += (Is - st->Is_prev[p][i]) * inv_dtp;
+                Mv += (Js - st->Js_prev[p][i]) * inv_dtp;
+            }
+            row[2 + 6 * p + i] = Fv;
+            row[5 + 6 * p + i] = Mv;
+            st->Is_prev[p][i] = Is;
+            st->Js_prev[p][i] = Js;
         }
-        row[2 + 6 * p + i] = Fv;
-        row[5 + 6 * p + i] = Mv;
-        st->Is_prev[p][i] = Is;
-        st->Js_prev[p][i] = Js;
-    }
-    __syncwarp();
-    const Frame& F = *fr;
-    if (tid < 2) {   // wing power at t^n (Sec. 3.5, Eq. insect_power)
-        const int s = tid;
-        double pa = 0.0, pi = 0.0;
-        if (s < ins->nwings) {
-            const double* m = row + 5 + 6 * (1 + s);
-            pa = -(m[0] * F.Ow[s][0] + m[1] * F.Ow[s][1] + m[2] * F.Ow[s][2]);
-            const double* J = ins->J_wing;   // xx yy zz xy xz yz
-            const M3 Jm = {{J[0], J[3], J[4], J[3], J[1], J[5], J[4], J[5], J[2]}};
-            const double* w = F.Oww[s];
-            double Jw[3], Jdw[3], c[3];
-            apply(Jm, w, Jw);
-            apply(Jm, F.dOww[s], Jdw);
-            cross3(w, Jw, c);
-            pi = w[0] * (Jdw[0] + c[0]) + w[1] * (Jdw[1] + c[1]) + w[2] * (Jdw[2] + c[2]);
+        __syncwarp();
+        const Frame& F = *fr;
+        if (tid < 2) {   // wing power at t^n (Sec. 3.5, Eq. insect_power)
+            const int s = tid;
+            double pa = 0.0, pi = 0.0;
+            if (s < ins->nwings) {
+                const double* m = row + 5 + 6 * (1 + s);
+                pa = -(m[0] * F.Ow[s][0] + m[1] * F.Ow[s][1] + m[2] * F.Ow[s][2]);
+                const double* J = ins->J_wing;   // xx yy zz xy xz yz
+                const M3 Jm = {{J[0], J[3], J[4], J[3], J[1], J[5], J[4], J[5], J[2]}};
+                const double* w = F.Oww[s];
+                double Jw[3], Jdw[3], c[3];
+                apply(Jm, w, Jw);
+                apply(Jm, F.dOww[s], Jdw);
+                cross3(w, Jw, c);
+                pi = w[0] * (Jdw[0] + c[0]) + w[1] * (Jdw[1] + c[1]) + w[2] * (Jdw[2] + c[2]);
+            }
+            row[22 + s] = pa;
+            row[24 + s] = pi;
         }
-        row[22 + s] = pa;
-        row[24 + s] = pi;
-    }
-    __syncwarp();
-    if (tid == 0) {
-        StepCoef c;
-        c.dt = dt;
-        c.n = n;
-        c.first = first;
-        c.t0 = st->t;
-        c.skip = 0;
-        if (first) {
-            c.c_now = dt;
-            c.c_old = 0.0;
-        } else {
-            double r = dt / dt_prev;
-            c.c_now = dt * (1.0 + 0.5 * r);
-            c.c_old = dt * 0.5 * r;
-        }
-        *coef = c;
-        row[0] = st->t;
-        row[1] = dt;
-        row[20] = 0.5 * tot[kSumEkin] * g.dx * g.dy * g.dz;
-        row[21] = umax;
+        __syncwarp();
+        if (tid == 0) {
+            StepCoef c;
+            c.dt = dt;
+            c.n = n;
+            c.first = first;
+            c.t0 = st->t;
+            c.skip = 0;
+            if (first) {
+                c.c_now = dt;
+                c.c_old = 0.0;
+            } else {
+                double r = dt / dt_prev;
+                c.c_now = dt * (1.0 + 0.5 * r);
+                c.c_old = dt * 0.5 * r;
+            }
+            *coef = c;
+            row[0] = st->t;
+            row[1] = dt;
+            row[20] = 0.5 * tot[kSumEkin] * g.dx * g.dy * g.dz;
+            row[21] = umax;
 
-        if (ins->free_flight) advance_body(ins, st, F, row, dt, first ? 0.0 : dt / dt_prev, first);
+            if (ins->free_flight) advance_body(ins, st, F, row, dt, first ? 0.0 : dt / dt_prev, first);
 
-        st->t += dt;
-        st->dt_prev = dt;
-        st->n = n + 1;
+            st->t += dt;
+            st->dt_prev = dt;
+            st->n = n + 1;
+        }
     }
+    cluster.sync();   // every CTA has read the others' sums
 }
 
 }  // namespace flusi
