@@ -291,6 +291,18 @@ struct StepState {
     double pad2;
 };
 
+// Whether this block leaves at entry: a device-side failure was recorded in the
+// status word (of st, or err where a TMA wait reports without a step state).
+// One answer for the whole block: the word can be written while blocks of a
+// kernel start (by the scalar kernel beside the forward passes, by a block whose
+// wait gave up), and a block that lost only some of its threads would go on with
+// tables and barriers those threads never set up.  Every thread calls it.
+__device__ __forceinline__ bool block_leaves(const StepState* st, const int* err)
+{
+    const bool gone = (st && *(volatile const int*)&st->status != 0) || (err && *(volatile const int*)err != 0);
+    return __syncthreads_or(gone) != 0;
+}
+
 // Coefficients of the current step, written by the scalar kernel and read by
 // the spectral update.
 struct StepCoef {

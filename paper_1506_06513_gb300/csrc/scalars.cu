@@ -481,17 +481,16 @@ k_scalars(Geom g, const double* part, int nparts, StepState* st, StepCoef* coef,
     __shared__ double own[kNumSums];
     __shared__ double tot[kNumSums];
     __shared__ double sh_dt;
+    __shared__ int saw, any_saw;
     const int tid = threadIdx.x, T = blockDim.x;
 
     // every thread of the cluster reads the state before the first cluster
-    // barrier; rank 0's thread 0 writes it only after that
-    const int status = st->status;
+    // barrier; rank 0's thread 0 writes it only after that.  A block of a pass
+    // beside this kernel may record a failure meanwhile: what each CTA's thread
+    // 0 saw is exchanged with the sums, so that the cluster goes one way.
     const long long n = st->n;
     const double dt_prev = st->dt_prev;
-    if (status != 0) {
-        if (rank == 0 && tid == 0) coef->skip = 1;
-        return;   // the whole cluster
-    }
+    if (tid == 0) saw = *(volatile int*)&st->status;
     // slot k, segment s of this CTA: the partials of CTAs [s c, (s + 1) c) in
     // order; then the segments in order
     if (tid < kNumSums * kScalarSeg) {
@@ -523,12 +522,16 @@ k_scalars(Geom g, const double* part, int nparts, StepState* st, StepCoef* coef,
             a = is_max ? fmax(a, v) : a + v;
         }
         tot[tid] = a;
+    } else if (tid == kNumSums) {
+        int a = 0;
+        for (int r = 0; r < kScalarCtas; ++r) a |= *cluster.map_shared_rank(&saw, r);
+        any_saw = a;
     }
     __syncthreads();
 
-    if (tot[kSumBad] != 0.0) {
+    if (any_saw != 0 || tot[kSumBad] != 0.0) {
         if (rank == 0 && tid == 0) {
-            st->status = FLUSI_ENONFINITE;
+            if (any_saw == 0) atomicCAS(&st->status, 0, (int)FLUSI_ENONFINITE);
             coef->skip = 1;
         }
         cluster.sync();   // the others have read this CTA's sums

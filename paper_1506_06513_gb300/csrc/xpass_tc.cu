@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 k_xpass_tc(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XExtra ex,
            const StepState* __restrict__ st)
 {
-    if (st && st->status != 0) return;
+    if (block_leaves(st, nullptr)) return;
     using Lt = TcLayout<Q, P>;
     constexpr int NH = Lt::NH, RB = Lt::RB, G = 16 / Q;   // G: 8-line groups of the 16-row stages
     constexpr int S = Lt::kSlots;

@@ -38,9 +38,8 @@ k_ypass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
         st = mb[blockIdx.z].st;
         err = &mb[blockIdx.z].st->status;
     }
-    if (st && st->status != 0) return;
     // after a TMA wait gave up, the remaining blocks leave at once
-    if (TMA && *(volatile int*)err != 0) return;
+    if (block_leaves(st, TMA ? err : nullptr)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int TX = 1 << lgTX, lgC = lgTX + lgNP, C = 1 << lgC;
     // the tile at a 128-byte boundary of shared memory (TMA destinations)

@@ -224,8 +224,7 @@ k_zinv(const cplx<T>* __restrict__ U, cplx<T>* __restrict__ W, Geom g, FftPlan p
         st = mb[blockIdx.z].st;
         err = &mb[blockIdx.z].st->status;
     }
-    if (st && st->status != 0) return;
-    if (TMA && *(volatile int*)err != 0) return;   // a TMA wait gave up earlier
+    if (block_leaves(st, TMA ? err : nullptr)) return;   // failed, or a TMA wait gave up earlier
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int TX = 1 << lgTX;
     // the tile at a 128-byte boundary of shared memory (TMA destinations)
@@ -401,8 +400,7 @@ k_zfwd(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict_
         st = mb[blockIdx.z].st;
         err = &mb[blockIdx.z].st->status;
     }
-    if (st && st->status != 0) return;
-    if (TMA && *(volatile int*)err != 0) return;   // a TMA wait gave up earlier
+    if (block_leaves(st, TMA ? err : nullptr)) return;   // failed, or a TMA wait gave up earlier
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int TX = 1 << lgTX;
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
