@@ -58,6 +58,10 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C b)
     return r;
 }
 
+// SMs of the GB300: a pass whose widest tiles would leave some without a block
+// takes narrower ones.
+constexpr int kSMs = 152;
+
 // Largest FFT length along any axis (the x transform runs at nx/2).
 constexpr int kMaxN = 1024;
 constexpr int kMaxStages = 10;

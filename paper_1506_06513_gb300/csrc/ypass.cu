@@ -261,6 +261,11 @@ template <typename T> YTile y_tile(const Geom& g, int ncomp)
     while (TX > 1 && (g.ny * TX > cap || TX > cmax)) TX >>= 1;
     int NP = 1;
     while (2 * NP * TX * g.ny <= cap && 2 * NP * TX <= std::min(kThreads, cmax) && 2 * NP <= g.nz) NP *= 2;
+    // small grids: fewer planes per tile until every SM has a block of a
+    // three-field pass (rows stay 128 bytes; one tile for every pass of a grid,
+    // as its tensor maps are)
+    const long long runs = (long long)current_batch().n * ceil_div(g.Mxp, TX) * 3;
+    while (NP > 1 && runs * ceil_div(g.nz, NP) < kSMs) NP >>= 1;
     t.lgTX = __builtin_ctz(TX);
     t.lgNP = __builtin_ctz(NP);
     t.blocks = ceil_div(g.Mxp, TX) * ceil_div(g.nz, NP) * ncomp;

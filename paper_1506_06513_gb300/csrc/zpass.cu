@@ -625,14 +625,24 @@ k_zupdate(const cplx<T>* __restrict__ Wn, cplx<T>* __restrict__ U, cplx<T>* __re
     }
 }
 
-template <typename T> int zinv_tx(const Geom& g)
+// Columns of a tile: the widest that fits, but on small grids narrower ones
+// (down to 32-byte rows, which L2 holds) until every SM has a block of the pass,
+// which takes `fields` tiles per column range.  The inverse pass handles a
+// column range in one block, a serial chain of five transforms (zinv at 128^3
+// FP32: 59 tiles of 64 columns 35 us, 234 of 16 24 us; at 32^3 FP64 4 tiles
+// 67 us, 126 of 2 columns 52 us); the forward pass has a block per field.
+template <typename T> int z_tx(const Geom& g, int fields)
 {
     const int cmax = g.zcols > 0 ? g.zcols : 64;   // columns per tile
     int TX = sizeof(T) == 4 ? 16 : 8;
     while (TX > 1 && (g.nz * TX > cap_zi<T>() || TX > cmax)) TX >>= 1;
     while (2 * TX * g.nz <= cap_zi<T>() && 2 * TX <= cmax) TX *= 2;
+    const long long tiles = (long long)current_batch().n * fields;
+    while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(g.My * g.Mxp, TX) < kSMs) TX >>= 1;
     return TX;
 }
+template <typename T> int zinv_tx(const Geom& g) { return z_tx<T>(g, 1); }
+template <typename T> int zfwd_tx(const Geom& g) { return z_tx<T>(g, 3); }
 
 template <typename T>
 cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan, const double2* tw,
@@ -665,7 +675,7 @@ cudaError_t launch_zf(void* W, int nf, const Geom& g, const FftPlan& plan, const
                       const int* pos, const StepState* st, const CUtensorMap* map, int bh, int* err,
                       cudaStream_t s)
 {
-    const int TX = zinv_tx<T>(g);
+    const int TX = zfwd_tx<T>(g);
     if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0 || nf < 1 || nf > 6) return cudaErrorInvalidValue;
     const int blocks = nf * ceil_div(g.My * g.Mxp, TX);
     const size_t smem = sizeof(cplx<T>) * ((size_t)g.nz + (size_t)g.nz * TX) + sizeof(rowidx_t) * g.nz + 128;
@@ -697,11 +707,10 @@ template <typename T> cudaError_t prepare_z(void* U, void* Ut, void* W, const Ge
     m->u_bh = m->ut_bh = m->w_bh = 0;
     const TensorMapEncoder encode = tensor_map_encoder();
     if (!encode) return cudaSuccess;   // no encoder: 16-byte copies
-    const int TX = zinv_tx<T>(g);
-    const size_t row_bytes = (size_t)TX * sizeof(cplx<T>);
+    const int TXi = zinv_tx<T>(g), TXf = zfwd_tx<T>(g);
     const size_t Q = (size_t)g.My * g.Mxp;
     const CUtensorMapDataType dt = sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-    auto make = [&](CUtensorMap* map, void* base, size_t rows, size_t ncomp, size_t rs, size_t cs, int bh) {
+    auto make = [&](CUtensorMap* map, void* base, size_t rows, size_t ncomp, size_t rs, size_t cs, int bh, int TX) {
         if (!base || bh <= 0 || bh > 256 || reinterpret_cast<uintptr_t>(base) % 16 != 0) return 0;
         const cuuint64_t dims[3] = {(cuuint64_t)(2 * Q), (cuuint64_t)rows, (cuuint64_t)ncomp};
         const cuuint64_t strides[2] = {(cuuint64_t)(rs * sizeof(cplx<T>)), (cuuint64_t)(cs * sizeof(cplx<T>))};
@@ -712,13 +721,13 @@ template <typename T> cudaError_t prepare_z(void* U, void* Ut, void* W, const Ge
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         return r == CUDA_SUCCESS ? bh : 0;
     };
-    const int ibh = inverse_box_rows(g.nz, g.Kz, row_bytes);
-    m->u_bh = make(&m->u, U, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh);
-    m->ut_bh = make(&m->ut, Ut, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh);
+    const int ibh = inverse_box_rows(g.nz, g.Kz, (size_t)TXi * sizeof(cplx<T>));
+    m->u_bh = make(&m->u, U, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
+    m->ut_bh = make(&m->ut, Ut, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
     int fbh = g.nz <= 256 ? g.nz : (g.nz % 256 == 0 ? 256 : 0);
-    if (((size_t)fbh * row_bytes) % 128 != 0) fbh = 0;
+    if (((size_t)fbh * TXf * sizeof(cplx<T>)) % 128 != 0) fbh = 0;
     const size_t Wplane = (size_t)g.ny * g.Mxp;
-    m->w_bh = make(&m->w, W, g.nz, 6, Wplane, (size_t)g.nz * Wplane, fbh);
+    m->w_bh = make(&m->w, W, g.nz, 6, Wplane, (size_t)g.nz * Wplane, fbh, TXf);
     return cudaSuccess;
 }
 
