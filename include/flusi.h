@@ -336,7 +336,9 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * stage in place of 4 4 or 8 2 (1024 = 16 8 8, 128 = 16 8, 16 = 16);
  * 2 fewest stages: as 1, and 2^(3q+2) with q >= 2 takes 16 16 in place of
  * 8 8 4 (256 = 16 16).  The inverse z pass always takes plan 0 (its kernel
- * has no radix-16 variant).
+ * has no radix-16 variant).  In FP32, plan 1 with the widest tiles takes the
+ * two-pass kernels (n = R L in two register passes) at the lengths that have
+ * them (most of 64..1024, z up to 512) in place of the radices reported.
  * Tile columns (y_cols, z_cols): 0 (default) the widest tile that fits a
  * block's 64 KB, else a cap on the tile's columns (x columns times z planes
  * for y; columns of the flattened (y, x) plane for z), a power of two of at

@@ -86,6 +86,7 @@ struct FftPlan {
     int mshift[kMaxStages];  // log2(m) when m is a power of two, else -1
     int ls[kMaxStages];      // block length radix*m
     int tstep[kMaxStages];   // twiddle index step (n/ls times the table stride)
+    int two_pass;            // FP32: the two-register-pass kernels where the length and tile have one (colfft.cuh)
 };
 
 // Grid and spectral truncation, shared by all kernels.
@@ -353,6 +354,15 @@ inline int inverse_box_rows(int n, int K, size_t row_bytes)
         if (k > 1 && ((size_t)bh * row_bytes) % 128 != 0) continue;
         return bh;
     }
+    return 0;
+}
+
+// Rows per TMA box for a forward tile of n rows: the largest divisor of n up to
+// 256 whose boxes start on 128-byte boundaries; 0 if there is none.
+inline int forward_box_rows(int n, size_t row_bytes)
+{
+    for (int bh = n < 256 ? n : 256; bh >= 8; --bh)
+        if (n % bh == 0 && (bh == n || ((size_t)bh * row_bytes) % 128 == 0)) return bh;
     return 0;
 }
 

@@ -125,6 +125,7 @@ FftPlan make_plan(int n, int tws, int mode = 0)
 {
     FftPlan p{};
     p.n = n;
+    p.two_pass = mode == 1;
     std::vector<int> r;
     int m = n;
     while (m % 3 == 0) { r.push_back(3); m /= 3; }
@@ -254,6 +255,7 @@ void layout(flusi_t h)
     // the inverse z pass holds more live values per thread (the curl's side
     // rows); a radix-16 stage there costs it a block per SM, more than it saves
     h->pzi = make_plan(h->nz, 1, 0);
+    h->pzi.two_pass = h->pz.two_pass;
     h->pyh = h->ny % 2 == 0 ? make_plan(h->ny / 2, 1, h->tune.y_plan) : FftPlan{};
     g.ycols = h->tune.y_cols;
     g.ypair = h->tune.y_pair;

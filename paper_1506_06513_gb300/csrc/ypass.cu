@@ -347,6 +347,13 @@ cudaError_t launch_y(bool inverse, void* W, const Geom& g, const FftPlan& plan, 
     YTile t = y_tile<T>(g, ncomp);
     if ((size_t)g.ny << (t.lgTX + t.lgNP) > (size_t)tile_elems<T>()) return cudaErrorInvalidValue;
     cplx<T>* w = (cplx<T>*)W;
+    if constexpr (sizeof(T) == 4) {
+        if (plan.two_pass && ycol_serves(g.ny, 1 << (t.lgTX + t.lgNP))) {
+            const int bh = maps && err && !current_batch().mb ? (inverse ? maps->inv_bh : maps->fwd_bh) : 0;
+            const CUtensorMap none{};
+            return launch_ycol(inverse, w, g, tw, ncomp, st, bh > 0 ? (inverse ? maps->inv : maps->fwd) : none, bh, err, s);
+        }
+    }
     return plan_has_radix16(plan) ? launch_y2<T, true>(inverse, w, g, plan, tw, pos, ncomp, st, maps, err, t, s)
                                   : launch_y2<T, false>(inverse, w, g, plan, tw, pos, ncomp, st, maps, err, t, s);
 }
@@ -377,9 +384,7 @@ template <typename T> cudaError_t prepare_y(void* W, const Geom& g, YMaps* m)
     // every box destination (row offsets of the tile) on a 128-byte boundary
     const size_t row_bytes = sizeof(cplx<T>) << (t.lgTX + t.lgNP);
     m->inv_bh = make(&m->inv, inverse_box_rows(g.ny, g.Ky, row_bytes));
-    int fbh = g.ny <= 256 ? g.ny : (g.ny % 256 == 0 ? 256 : 0);
-    if (((size_t)fbh * row_bytes) % 128 != 0) fbh = 0;
-    m->fwd_bh = make(&m->fwd, fbh);
+    m->fwd_bh = make(&m->fwd, forward_box_rows(g.ny, row_bytes));
     return cudaSuccess;
 }
 
@@ -428,7 +433,8 @@ int ypass_paired(int fp64, const Geom& g) { return fp64 ? y_paired<double>(g) : 
 cudaError_t configure_ypass()
 {
     const int big = 100 * 1024;
-    cudaError_t e;
+    cudaError_t e = configure_ycol();
+    if (e) return e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
 #define FLUSI_SMEM_Y(T, R16)                         \

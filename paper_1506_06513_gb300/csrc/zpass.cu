@@ -662,6 +662,10 @@ cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan
     // the inverse z pass is built without radix-16 stages (its plan has none)
     if (plan_has_radix16(plan)) return cudaErrorInvalidValue;
     const Batch& B = current_batch();
+    if constexpr (sizeof(T) == 4) {
+        if (plan.two_pass && zcol_serves(g.nz, TX) && (nf == 3 || nf == 6))
+            return launch_zcol_inv(u, w, g, tw, nf, st, m, tma && !B.mb ? bh : 0, err, s);
+    }
     const dim3 grid(blocks, 1, B.n);
     if (tma && !B.mb)
         k_zinv<T, true, false><<<grid, kThreadsInv, smem, s>>>(u, w, g, plan, tw, pos, nf, lg, st, m, bh, err, nullptr);
@@ -687,6 +691,9 @@ cudaError_t launch_zf(void* W, int nf, const Geom& g, const FftPlan& plan, const
     const Batch& B = current_batch();
     const dim3 grid(blocks, 1, B.n);
     const bool use_tma = tma && !B.mb;
+    if constexpr (sizeof(T) == 4) {
+        if (plan.two_pass && zcol_serves(g.nz, TX)) return launch_zcol_fwd(w, nf, g, tw, st, m, use_tma ? bh : 0, err, s);
+    }
     if (plan_has_radix16(plan)) {
         if (use_tma) k_zfwd<T, true, true><<<grid, kThreadsInv, smem, s>>>(w, g, plan, tw, pos, lg, st, m, bh, err, nullptr);
         else k_zfwd<T, false, true><<<grid, kThreadsInv, smem, s>>>(w, g, plan, tw, pos, lg, st, m, 0, err, B.mb);
@@ -724,8 +731,7 @@ template <typename T> cudaError_t prepare_z(void* U, void* Ut, void* W, const Ge
     const int ibh = inverse_box_rows(g.nz, g.Kz, (size_t)TXi * sizeof(cplx<T>));
     m->u_bh = make(&m->u, U, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
     m->ut_bh = make(&m->ut, Ut, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
-    int fbh = g.nz <= 256 ? g.nz : (g.nz % 256 == 0 ? 256 : 0);
-    if (((size_t)fbh * TXf * sizeof(cplx<T>)) % 128 != 0) fbh = 0;
+    const int fbh = forward_box_rows(g.nz, (size_t)TXf * sizeof(cplx<T>));
     const size_t Wplane = (size_t)g.ny * g.Mxp;
     m->w_bh = make(&m->w, W, g.nz, 6, Wplane, (size_t)g.nz * Wplane, fbh, TXf);
     return cudaSuccess;
@@ -848,7 +854,8 @@ cudaError_t launch_divergence(int fp64, const void* U, const Geom& g, unsigned l
 cudaError_t configure_zpass()
 {
     const int big = 120 * 1024;
-    cudaError_t e;
+    cudaError_t e = configure_zcol();
+    if (e) return e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
 #define FLUSI_SMEM_Z(T, R16)                  \
