@@ -11,7 +11,7 @@ const XLineOps* xline_table_medium(int* n)
         XLineOf<XLine<12, 8, 4>>::all(),
         XLineOf<XLine<18, 6, 5>>::all(),
         XLineOf<XLine<12, 12, 2>>::all(),
-        XLineOf<XLine<16, 8, 4>>::lines_only(),
+        XLineOf<XLine<16, 8, 4>>::all(),
     };
     *n = int(sizeof t / sizeof t[0]);
     return t;

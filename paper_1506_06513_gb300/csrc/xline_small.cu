@@ -15,9 +15,9 @@ const XLineOps* xline_table_small(int* n)
         XLineOf<XLine<9, 3, 10>>::all(),
         XLineOf<XLine<6, 6, 5>>::all(),
         XLineOf<XLine<9, 6, 5>>::all(),
-        XLineOf<XLine<8, 4, 8>>::lines_only(),
+        XLineOf<XLine<8, 4, 8>>::all(),
         XLineOf<XLine<12, 4, 8>>::lines_only(),
-        XLineOf<XLine<8, 8, 4>>::lines_only(),
+        XLineOf<XLine<8, 8, 4>>::all(),
     };
     *n = int(sizeof t / sizeof t[0]);
     return t;

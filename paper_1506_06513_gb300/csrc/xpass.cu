@@ -1067,8 +1067,8 @@ template <typename T, int R, int S> size_t sq_smem(const Geom& g, bool sponge = 
     return s;
 }
 
-// grid = the virtual CTAs (rows of partial sums, x_grid); a batch of n
-// members runs about one resident wave in all, each CTA taking several
+// grid = the virtual CTAs (rows of partial sums, x_grid, whichever kernel it was
+// counted for); a batch of n members runs about one resident wave in all, each CTA taking several
 // virtual ones, instead of n full grids of CTAs that each take one or two
 // tiles and pay their table and frame loads for them.
 template <typename T, int R, int S>
@@ -1116,6 +1116,19 @@ template <typename T> int sq_kind(const Geom& g)
     }
 }
 
+// The general line kernel (xline.cuh) for the physical pass of this grid, or
+// nullptr.  Where a kernel above serves the length too, the measured faster one:
+// FP32 x pass of 256^3 227 us here and 170 there, 128^3 41 and 35, 64^3 27 and 25;
+// 512^3 1.13 ms here and 1.21 there, 1024^3 12.5 and 13.4, 96 x 96 x 192 37 and 39.
+// The sponge is fused only here.
+template <typename T> const XLineOps* phys_line(const Geom& g, bool sponge)
+{
+    const XLineOps* o = xline_of<T>(g);
+    if (!o || !o->phys) return nullptr;
+    const int kind = sq_kind<T>(g);
+    return kind == 0 || (!sponge && (kind == 80 || kind == 81 || kind == 82)) ? o : nullptr;
+}
+
 template <typename T> int x_lgrb(const Geom& g)
 {
     const int nh = g.nx / 2;
@@ -1139,12 +1152,15 @@ template <typename T> int x_grid(const Geom& g)
     const int sm_count = sm_count_here();
     int per_sm = 0, ntiles = 0;
     const int kind = sq_kind<T>(g);
-    const XLineOps* line = kind == 0 ? xline_of<T>(g) : nullptr;
+    const XLineOps* line = phys_line<T>(g, false);
 #define FLUSI_SQ_OCC(R, S)                                                                          \
     ntiles = ceil_div(g.nz * g.ny, sq_rows<sq_lanes<R, S>()>());                                               \
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, false>, 192, \
                                                   sq_smem<T, R, S>(g));
-    if (kind == 161) {
+    if (line) {
+        ntiles = ceil_div(g.nz * g.ny, line->rows);
+        per_sm = line->phys_per_sm();
+    } else if (kind == 161) {
         FLUSI_SQ_OCC(16, 1)
     } else if (kind == 81) {
         FLUSI_SQ_OCC(8, 1)
@@ -1156,9 +1172,6 @@ template <typename T> int x_grid(const Geom& g)
         FLUSI_SQ_OCC(12, 0)
     } else if (kind == 80) {
         FLUSI_SQ_OCC(8, 0)
-    } else if (line) {
-        ntiles = ceil_div(g.nz * g.ny, line->rows);
-        per_sm = line->phys_per_sm();
     } else {
         const int lg = x_lgrb<T>(g);
         ntiles = ceil_div(g.nz * g.ny, 1 << lg);
@@ -1191,7 +1204,7 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
             line->lines(mode, s, w, g, tw, ex, sm_count_here());
             return cudaGetLastError();
         }
-        if (line && line->phys && mode == XP_PHYS && sq_kind<T>(g) == 0) {
+        if (mode == XP_PHYS && phys_line<T>(g, sponge)) {
             const Batch& B = current_batch();
             XExtra e = ex;
             e.nvirt = x_grid<T>(g);
