@@ -338,9 +338,10 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * 8 8 4 (256 = 16 16).  The inverse z pass always takes plan 0 (its kernel
  * has no radix-16 variant).  In FP32, plan 1 with the widest tiles takes the
  * two-pass kernels (n = R L in two register passes) at the lengths that have
- * them (most of 64..1024, z up to 512) in place of the radices reported.
+ * them (most of 64..1024) in place of the radices reported.
  * Tile columns (y_cols, z_cols): 0 (default) the widest tile that fits a
- * block's 64 KB, else a cap on the tile's columns (x columns times z planes
+ * block's 64 KB (two-pass kernels over 512 rows: 16 columns, 128 KB; on grids
+ * whose widest tiles would not fill the GPU, a narrower one), else a cap on the tile's columns (x columns times z planes
  * for y; columns of the flattened (y, x) plane for z), a power of two of at
  * least 32 bytes of complex values (4 in FP32, 2 in FP64) and at most 256.
  * x_kernel: 0 (default) the register-resident line kernel where one exists

@@ -13,15 +13,19 @@
 //
 // The kernels are persistent: a block keeps its twiddle table and loops over
 // tiles, and as soon as pass 2 has read a tile the next one's copies go out into
-// its place.  Loads, not arithmetic, are what these passes wait for.  Radices up
-// to 18 leave registers for three blocks of 256 threads per SM, one tile each.
-// Larger ones leave two groups of 256 threads, but shared memory for three
-// tiles: they form one block of two groups over a ring of three tiles, each
-// group taking every second load, so that one tile is always on its way (y
-// inverse at 512^3: 0.68 ms as two blocks of one tile, 0.56 so).  Tiles of 8
-// columns stay two blocks of one tile: their 64-byte rows share 128-byte lines
-// with a neighbour's, and more of them in flight cost more than the overlap gives
-// (y inverse at 1024^3: 5.4 ms, 8.4 in the ring).
+// its place.  Loads, not arithmetic, are what these passes wait for.
+//   Radices up to 18 leave registers for three blocks of 256 threads per SM, one
+//   tile each.
+//   Larger ones leave two groups of 256 threads, but shared memory for three
+//   tiles: they form one block of two groups over a ring of three tiles, each
+//   group taking every second load, so that one tile is always on its way (y
+//   inverse at 512^3: 0.68 ms as two blocks of one tile, 0.56 so).
+//   Over 512 rows a 64 KB tile would have 8 columns, 64-byte rows that share
+//   128-byte lines with a neighbour's: such tiles in a ring took 8.4 ms for the y
+//   inverse at 1024^3, as two blocks 5.4 to 6.3, in the z inverse 7.8.  There a
+//   block of 512 threads takes 16 columns, 128 KB in two halves of the rows over a
+//   ring of three halves (the first half of the next tile flies while this one
+//   is transformed): 5.1 and 4.3 ms, the forward passes 2.3 and 1.7 (z staged 2.8).
 
 // A tile's rows are C consecutive values, so a warp's 8-byte accesses cover whole
 // 128-byte lines (C >= 16); with C = 8 (n > 512) pass 2 meets each bank twice.
@@ -33,25 +37,38 @@
 namespace flusi {
 namespace {
 
-constexpr int kColThreads = 256;   // of a group
-
-// columns of a full tile (64 KB of shared memory) of length n, at most `most`
+// columns of a full tile of length n (64 KB of shared memory; over 512 rows 16
+// columns), at most `most`
 constexpr int col_tile(int n, int most)
 {
     int c = 8;
-    while (2 * c * n <= 8192 && 2 * c <= most) c *= 2;
+    while (2 * c * n <= (n > 512 ? 16384 : 8192) && 2 * c <= most) c *= 2;
     return c;
 }
 
 template <int R_, int L_, int C_> struct Col {
-    static constexpr int R = R_, L = L_, C = C_, N = R * L, T = kColThreads;
+    static constexpr int R = R_, L = L_, C = C_, N = R * L;
+    static constexpr int CH = N > 512 ? 2 : 1;                 // loads (row ranges) of a tile
+    static constexpr int T = CH == 2 ? 512 : 256;              // threads of a group
     static constexpr int U1 = L * C, U2 = R * C;               // threads' work items of the passes
     static constexpr int ROUNDS1 = (U1 + T - 1) / T, ROUNDS2 = (U2 + T - 1) / T;
     static constexpr bool SMALL = R <= 18 && L <= 18;
-    static constexpr int GROUPS = SMALL || C == 8 ? 1 : 2, BUFS = GROUPS == 1 ? 1 : 3;
-    static constexpr int THREADS = GROUPS * T, MINB = GROUPS == 2 ? 1 : SMALL ? 3 : 2;
-    static constexpr size_t kSmem = sizeof(float2) * ((size_t)BUFS * N * C + N) + 128;
-    static_assert((C & (C - 1)) == 0 && N * C <= 8192, "a tile");
+    static constexpr int GROUPS = SMALL || CH == 2 ? 1 : 2, BUFS = SMALL ? 1 : 3;
+    static constexpr int THREADS = GROUPS * T, MINB = SMALL ? 3 : 1;
+    static constexpr int BUF = N * C / CH;                     // values of a buffer
+    static constexpr size_t kSmem = sizeof(float2) * ((size_t)BUFS * BUF + N) + 128;
+    static_assert((C & (C - 1)) == 0 && BUF <= 8192 && (CH == 1 || (R % 2 == 0 && !SMALL)), "a tile");
+
+    // A tile: the buffer of its rows, or of its first and its second half of rows.
+    struct Tile {
+        float2 *lo, *hi;
+        // row range q of L rows (q < R)
+        __device__ __forceinline__ float2* rows(int q) const
+        {
+            if constexpr (CH == 1) return lo + q * L * C;
+            else return q < R / 2 ? lo + q * L * C : hi + (q - R / 2) * L * C;
+        }
+    };
 
     // rows [lo, hi] of a transform that keeps |m| <= K, K = N/3 or (strict rule,
     // N divisible by 3) N/3 - 1: 0 all dropped, 2 all kept, 1 it depends
@@ -72,30 +89,29 @@ template <int R_, int L_, int C_> struct Col {
     // pass 1; PRUNED: rows of dropped modes are zero (whatever the tile holds
     // there); weigh(v, row) may scale an input
     template <bool INV, bool PRUNED, class Weigh>
-    __device__ __forceinline__ static void first(float2* buf, const float2* tws, int tid, int K, Weigh weigh)
+    __device__ __forceinline__ static void first(const Tile& tile, const float2* tws, int tid, int K, Weigh weigh)
     {
 #pragma unroll 1
         for (int rd = 0; rd < ROUNDS1; ++rd) {
             const int u = tid + rd * T;
             if (U1 % T != 0 && u >= U1) break;
             const int j = u / C;
-            float2* p = buf + u;                      // row j, column u % C
-            float2 v[R];
+            float2 v[R];                              // rows j + L t of column u % C
 #pragma unroll
             for (int t = 0; t < R; ++t) {
                 const int k = PRUNED ? kept(L * t, L * t + L - 1) : 2;
                 const int row = j + L * t;
                 if (k == 0) v[t] = make_float2(0.0f, 0.0f);
-                else if (k == 2) v[t] = weigh(p[t * L * C], row);
-                else v[t] = row <= K || row >= N - K ? weigh(p[t * L * C], row) : make_float2(0.0f, 0.0f);
+                else if (k == 2) v[t] = weigh(tile.rows(t)[u], row);
+                else v[t] = row <= K || row >= N - K ? weigh(tile.rows(t)[u], row) : make_float2(0.0f, 0.0f);
             }
             Dft<float, R, INV>::run(v);
-            p[0] = v[0];
+            tile.rows(0)[u] = v[0];
 #pragma unroll
             for (int q = 1; q < R; ++q) {
                 float2 w = tws[q * L + j];
                 if (INV) w.y = -w.y;
-                p[q * L * C] = cmul(v[q], w);
+                tile.rows(q)[u] = cmul(v[q], w);
             }
         }
     }
@@ -104,7 +120,7 @@ template <int R_, int L_, int C_> struct Col {
     // with a[i] the value of frequency q + R i; refill() once every value is
     // read.  Every thread of the group calls it.
     template <bool INV, class Io, class Refill>
-    __device__ __forceinline__ static void second(const float2* buf, int tid, Io& io, Refill refill)
+    __device__ __forceinline__ static void second(const Tile& tile, int tid, Io& io, Refill refill)
     {
 #pragma unroll 1
         for (int rd = 0; rd < ROUNDS2; ++rd) {
@@ -114,7 +130,7 @@ template <int R_, int L_, int C_> struct Col {
             float2 a[L];
             if (on) {
                 io.begin(q, col);
-                const float2* p = buf + q * L * C + col;
+                const float2* p = tile.rows(q) + col;
 #pragma unroll
                 for (int i = 0; i < L; ++i) a[i] = p[i * C];
             }
@@ -129,20 +145,20 @@ template <int R_, int L_, int C_> struct Col {
 
 // barriers of one group of threads: all of it meets, or the first warp waits
 // for the others (who do not wait).  Ids 1 and 2 for group 0, 3 and 4 for group 1.
-__device__ __forceinline__ void group_sync(int group)
+template <int T> __device__ __forceinline__ void group_sync(int group)
 {
-    if (group == 0) asm volatile("bar.sync 1, %0;" ::"n"(kColThreads) : "memory");
-    else asm volatile("bar.sync 3, %0;" ::"n"(kColThreads) : "memory");
+    if (group == 0) asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+    else asm volatile("bar.sync 3, %0;" ::"n"(T) : "memory");
 }
-__device__ __forceinline__ void group_gather(int group)
+template <int T> __device__ __forceinline__ void group_gather(int group)
 {
-    if (group == 0) asm volatile("bar.sync 2, %0;" ::"n"(kColThreads) : "memory");
-    else asm volatile("bar.sync 4, %0;" ::"n"(kColThreads) : "memory");
+    if (group == 0) asm volatile("bar.sync 2, %0;" ::"n"(T) : "memory");
+    else asm volatile("bar.sync 4, %0;" ::"n"(T) : "memory");
 }
-__device__ __forceinline__ void group_report(int group)
+template <int T> __device__ __forceinline__ void group_report(int group)
 {
-    if (group == 0) asm volatile("bar.arrive 2, %0;" ::"n"(kColThreads) : "memory");
-    else asm volatile("bar.arrive 4, %0;" ::"n"(kColThreads) : "memory");
+    if (group == 0) asm volatile("bar.arrive 2, %0;" ::"n"(T) : "memory");
+    else asm volatile("bar.arrive 4, %0;" ::"n"(T) : "memory");
 }
 
 struct ColState {
@@ -151,11 +167,12 @@ struct ColState {
     int bad[2];                   // per group: a wait gave up
 };
 
-// The loads of a block, numbered 0, 1, 2, ...: load i lands in buffer i % BUFS,
-// as that buffer's load number i / BUFS, and belongs to group i % GROUPS.
-// Job: bool exists(i) (false from some i on), issue(i, buf, bar) by one thread
-// (TMA boxes, after an expect_tx) or copy(i, buf, tid) by a group's threads
-// (16-byte copies), work(i, buf, tid, group, refill).
+// The tiles of a block, numbered 0, 1, 2, ...: tile i belongs to group i % GROUPS
+// and takes the loads i CH + h, h < CH (its row ranges).  Load s lands in buffer
+// s % BUFS, as that buffer's load number s / BUFS.
+// Job: bool exists(i) (false from some i on), issue(i, h, buf, bar) by one thread
+// (TMA boxes, after an expect_tx) or copy(i, h, buf, tid) by a group's threads
+// (16-byte copies), work(i, tile, tid, group, refill).
 //
 // A buffer's barrier tells two loads apart only by parity, so a group first
 // waits until its load has been sent (the one before it in that buffer has then
@@ -167,19 +184,20 @@ template <class X, class Job>
 __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, int* err, Job& job)
 {
     constexpr long long kLimit = 400000000LL;   // SM clocks, as mbar_wait
+    constexpr int CH = X::CH;
     const int group = X::GROUPS == 1 ? 0 : (threadIdx.x >= X::T ? 1 : 0), tid = threadIdx.x & (X::T - 1);
-    auto slot_of = [](int i) { return X::BUFS == 1 ? 0 : i % X::BUFS; };
-    auto buffer = [&](int i) { return bufs + slot_of(i) * (X::N * X::C); };
-    auto sent = [&](int i) { *(volatile int*)&sh.issued[slot_of(i)] = i / X::BUFS + 1; };
-    auto send = [&](int i) {      // one thread
-        job.issue(i, buffer(i), sh.full + slot_of(i));
-        sent(i);
+    auto slot_of = [](int s) { return X::BUFS == 1 ? 0 : s % X::BUFS; };
+    auto buffer = [&](int s) { return bufs + slot_of(s) * X::BUF; };
+    auto sent = [&](int s) { *(volatile int*)&sh.issued[slot_of(s)] = s / X::BUFS + 1; };
+    auto send = [&](int s) {      // one thread
+        job.issue(s / CH, s % CH, buffer(s), sh.full + slot_of(s));
+        sent(s);
     };
-    auto copy_in = [&](int i) {   // the group's threads; each arrives when its copies have landed
-        job.copy(i, buffer(i), tid);
-        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(sh.full + slot_of(i)))
+    auto copy_in = [&](int s) {   // the group's threads; each arrives when its copies have landed
+        job.copy(s / CH, s % CH, buffer(s), tid);
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(sh.full + slot_of(s)))
                      : "memory");
-        if (tid == 0) sent(i);
+        if (tid == 0) sent(s);
     };
     if (threadIdx.x == 0) {
         for (int b = 0; b < X::BUFS; ++b) {
@@ -191,42 +209,48 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
     __syncthreads();   // the state (and the caller's tables) are set
     if (tma) {
         if (threadIdx.x == 0)
-            for (int i = 0; i < X::BUFS; ++i)
-                if (job.exists(i)) send(i);
+            for (int s = 0; s < X::BUFS; ++s)
+                if (job.exists(s / CH)) send(s);
     } else if (group == 0) {
-        for (int i = 0; i < X::BUFS; ++i)
-            if (job.exists(i)) copy_in(i);
+        for (int s = 0; s < X::BUFS; ++s)
+            if (job.exists(s / CH)) copy_in(s);
     }
 #pragma unroll 1
     for (int i = group; job.exists(i); i += X::GROUPS) {
-        const int load = i / X::BUFS;
         bool ok = true;
-        const long long t0 = clock64();
-        while (ok && *(volatile int*)&sh.issued[slot_of(i)] <= load) ok = clock64() - t0 <= kLimit;
-        if (ok) ok = mbar_wait(sh.full + slot_of(i), (unsigned)load & 1u, kLimit);
+#pragma unroll
+        for (int h = 0; h < CH; ++h) {
+            const int s = i * CH + h, load = s / X::BUFS;
+            const long long t0 = clock64();
+            while (ok && *(volatile int*)&sh.issued[slot_of(s)] <= load) ok = clock64() - t0 <= kLimit;
+            if (ok) ok = mbar_wait(sh.full + slot_of(s), (unsigned)load & 1u, kLimit);
+        }
         if (!ok) {
             *(volatile int*)&sh.bad[group] = 1;
             atomicCAS(err, 0, (int)FLUSI_ETIMEOUT);
         }
         __syncwarp();
-        group_sync(group);
+        group_sync<X::T>(group);
         if (*(volatile int*)&sh.bad[group]) break;   // only this group sets it, before the barrier
-        const int next = i + X::BUFS;
-        job.work(i, buffer(i), tid, group, [&] {
-            // the group has read the tile: refill it
-            if (!job.exists(next)) return;
+        const int next = i * CH + X::BUFS;
+        typename X::Tile tile{buffer(i * CH), buffer(i * CH + CH - 1)};
+        job.work(i, tile, tid, group, [&] {
+            // the group has read the tile: refill its buffers
+            if (!job.exists(next / CH)) return;
             if (!tma) {
-                group_sync(group);
-                copy_in(next);
+                group_sync<X::T>(group);
+                for (int h = 0; h < CH; ++h)
+                    if (job.exists((next + h) / CH)) copy_in(next + h);
             } else if (tid < 32) {
-                group_gather(group);
+                group_gather<X::T>(group);
                 if (tid == 0) {
                     fence_proxy_async();   // the generic accesses to the tile before the asynchronous proxy's
-                    send(next);
+                    for (int h = 0; h < CH; ++h)
+                        if (job.exists((next + h) / CH)) send(next + h);
                 }
                 __syncwarp();
             } else {
-                group_report(group);
+                group_report<X::T>(group);
             }
         });
     }
@@ -237,15 +261,12 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
 }
 
 // The lengths served, X(n, R, L).  Others (and narrowed tiles, the other plans
-// and FP64) take the staged kernels of ypass.cu and zpass.cu, and so do the z
-// passes over 512: with 8 columns a tile the two-pass inverse is slower there
-// (1024^3: 7.8 ms against 6.5, its side rows need more registers than are left).
-#define FLUSI_COL_SHORT(X)                                                                                 \
+// and FP64) take the staged kernels of ypass.cu and zpass.cu.
+#define FLUSI_COL_LENGTHS(X)                                                                               \
     X(64, 8, 8) X(72, 9, 8) X(81, 9, 9) X(96, 12, 8) X(108, 12, 9) X(128, 16, 8) X(144, 12, 12)            \
     X(162, 18, 9) X(192, 16, 12) X(216, 18, 12) X(243, 27, 9) X(256, 16, 16) X(288, 18, 16) X(324, 18, 18) \
-    X(384, 24, 16) X(432, 27, 16) X(486, 27, 18) X(512, 32, 16)
-#define FLUSI_COL_LENGTHS(X) \
-    FLUSI_COL_SHORT(X) X(576, 24, 24) X(648, 27, 24) X(768, 32, 24) X(864, 32, 27) X(1024, 32, 32)
+    X(384, 24, 16) X(432, 27, 16) X(486, 27, 18) X(512, 32, 16) X(576, 24, 24) X(648, 24, 27)              \
+    X(768, 32, 24) X(864, 32, 27) X(1024, 32, 32)
 
 inline int col_sms()
 {

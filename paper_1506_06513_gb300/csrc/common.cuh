@@ -102,6 +102,8 @@ struct Geom {
     // z tile, the shared-memory x kernel in place of the line kernel, and the
     // paired (two-CTA) y kernel where ny is even
     int ycols, zcols, xgeneric, ypair;
+    // y and z plans that take the two-pass kernels where they exist (FP32)
+    int two_pass_y, two_pass_z;
     // physical x pass on the tensor cores with the operands split into xtc
     // BF16 pieces (2 or 3); 0: FP32 (or FP64) arithmetic units
     int xtc;

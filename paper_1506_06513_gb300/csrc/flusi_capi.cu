@@ -257,6 +257,8 @@ void layout(flusi_t h)
     h->pzi = make_plan(h->nz, 1, 0);
     h->pzi.two_pass = h->pz.two_pass;
     h->pyh = h->ny % 2 == 0 ? make_plan(h->ny / 2, 1, h->tune.y_plan) : FftPlan{};
+    g.two_pass_y = h->py.two_pass;
+    g.two_pass_z = h->pz.two_pass;
     g.ycols = h->tune.y_cols;
     g.ypair = h->tune.y_pair;
     g.zcols = h->tune.z_cols;

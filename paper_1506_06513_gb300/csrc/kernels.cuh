@@ -65,6 +65,7 @@ cudaError_t launch_ypass(int fp64, bool inverse, void* W, const Geom& g, const F
                          const YMaps* maps, int* err, cudaStream_t s, const FftPlan* half = nullptr,
                          const int* pos_half = nullptr);
 // the two-register-pass y and z kernels (ycol.cu, zcol.cu)
+// a length and tile width served; over 512 rows their tiles have twice the columns
 bool zcol_serves(int nz, int cols);
 cudaError_t launch_zcol_fwd(float2* W, int nf, const Geom& g, const double2* tw, const StepState* st, const CUtensorMap& map,
                             int bh, int* err, cudaStream_t s);

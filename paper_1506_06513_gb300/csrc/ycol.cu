@@ -1,17 +1,16 @@
 // y passes in two register passes (colfft.cuh): the FP32 y transforms of
-// ypass.cu at the lengths of FLUSI_COL_LENGTHS, full tiles.  A tile is TX
-// consecutive x modes (128-byte rows, 64 for n > 512) of NP consecutive z planes
-// of one component.
+// ypass.cu at the lengths of FLUSI_COL_LENGTHS, full tiles.  A tile is 16
+// consecutive x modes of NP consecutive z planes of one component.
 #include "colfft.cuh"
 
 namespace flusi {
 namespace {
 
 template <int N> constexpr int y_cols() { return col_tile(N, 256); }
-template <int N> constexpr int y_tx() { return y_cols<N>() < 16 ? 8 : 16; }
+constexpr int kTX = 16;   // x modes of a tile, 128-byte rows
 
 template <class X, bool INV> struct YJob {
-    static constexpr int C = X::C, N = X::N, R = X::R, TX = y_tx<N>(), NP = C / TX;
+    static constexpr int C = X::C, N = X::N, R = X::R, TX = kTX, NP = C / TX;
     float2* W;
     const float2* tws;
     const CUtensorMap* map;
@@ -27,41 +26,43 @@ template <class X, bool INV> struct YJob {
         c = b / nzb;
         z0 = (b - c * nzb) * NP;
     }
-    // boxes of bh rows of NP planes of TX columns.  Inverse: modes 0..Ky to
-    // rows 0..Ky, modes Ky..2Ky to rows N-Ky-1..N-1 (row N-Ky-1, a dropped
-    // mode, is not read).
-    __device__ __forceinline__ void issue(int i, float2* buf, unsigned long long* bar) const
+    // boxes of bh rows of NP planes of TX columns: rows h N/CH to (h+1) N/CH.
+    // Inverse: modes 0..Ky to rows 0..Ky, modes Ky..2Ky to rows N-Ky-1..N-1 (row
+    // N-Ky-1, a dropped mode, is not read).
+    __device__ __forceinline__ void issue(int i, int h, float2* buf, unsigned long long* bar) const
     {
+        constexpr int CH = X::CH, half = N / CH;
         int x0, z0, c;
         where(i, x0, z0, c);
         const int pl = c * nz + z0;
         const unsigned box = (unsigned)(bh * C * sizeof(float2));
         if (INV) {
             const int kb = (Ky + 1) / bh;
-            mbar_expect_tx(bar, 2 * kb * box);
+            mbar_expect_tx(bar, (CH == 1 ? 2 : 1) * kb * box);
             for (int q = 0; q < kb; ++q) {
-                tma_load_3d(buf + q * bh * C, map, 2 * x0, pl, q * bh, bar);
-                tma_load_3d(buf + (N - Ky - 1 + q * bh) * C, map, 2 * x0, pl, Ky + q * bh, bar);
+                if (CH == 1 || h == 0) tma_load_3d(buf + q * bh * C, map, 2 * x0, pl, q * bh, bar);
+                if (CH == 1 || h == 1)
+                    tma_load_3d(buf + ((CH == 1 ? N : half) - Ky - 1 + q * bh) * C, map, 2 * x0, pl, Ky + q * bh, bar);
             }
         } else {
-            const int nb = N / bh;
+            const int nb = half / bh;
             mbar_expect_tx(bar, nb * box);
-            for (int q = 0; q < nb; ++q) tma_load_3d(buf + q * bh * C, map, 2 * x0, pl, q * bh, bar);
+            for (int q = 0; q < nb; ++q) tma_load_3d(buf + q * bh * C, map, 2 * x0, pl, h * half + q * bh, bar);
         }
     }
     // the same rows by 16-byte copies, two columns each (columns outside the
     // grid are left as they are: nothing of them is stored)
-    __device__ __forceinline__ void copy(int i, float2* buf, int tid) const
+    __device__ __forceinline__ void copy(int i, int h, float2* buf, int tid) const
     {
         int x0, z0, c;
         where(i, x0, z0, c);
-        constexpr int lanes = C / 2;
+        constexpr int lanes = C / 2, half = N / X::CH;
         const int col = (tid % lanes) * 2, z = z0 + col / TX, x = x0 + col % TX;
         if (z >= nz || x >= Mxp) return;   // Mxp is a multiple of 4
         const float2* src = W + ((size_t)c * nz + z) * plane + x;
-        for (int s = tid / lanes; s < N; s += X::T / lanes) {
-            const int j = INV ? (s <= Ky ? s : (s >= N - Ky ? s - N + My : -1)) : s;
-            if (j >= 0) cp_async_16(buf + s * C + col, src + (size_t)j * Mxp);
+        for (int o = tid / lanes; o < half; o += X::T / lanes) {
+            const int s = h * half + o, j = INV ? (s <= Ky ? s : (s >= N - Ky ? s - N + My : -1)) : s;
+            if (j >= 0) cp_async_16(buf + o * C + col, src + (size_t)j * Mxp);
         }
     }
     struct Io {
@@ -95,14 +96,14 @@ template <class X, bool INV> struct YJob {
         }
     };
     template <class Refill>
-    __device__ __forceinline__ void work(int i, float2* buf, int tid, int group, Refill refill) const
+    __device__ __forceinline__ void work(int i, const typename X::Tile& t, int tid, int group, Refill refill) const
     {
         int x0, z0, c;
         where(i, x0, z0, c);
-        X::template first<INV, INV>(buf, tws, tid, Ky, [](float2 v, int) { return v; });
-        group_sync(group);
+        X::template first<INV, INV>(t, tws, tid, Ky, [](float2 v, int) { return v; });
+        group_sync<X::T>(group);
         Io io{*this, W + (size_t)c * nz * plane, x0, z0, 0, nullptr, false};
-        X::template second<INV>(buf, tid, io, refill);
+        X::template second<INV>(t, tid, io, refill);
     }
 };
 
@@ -122,7 +123,7 @@ k_ycol(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, int ncomp
     __shared__ ColState state;
     // the tiles at a 128-byte boundary of shared memory (TMA destinations)
     float2* bufs = reinterpret_cast<float2*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
-    float2* tws = bufs + X::BUFS * X::N * X::C;
+    float2* tws = bufs + X::BUFS * X::BUF;
     using Job = YJob<X, INV>;
     const int nxb = ceil_div(g.Mxp, Job::TX), nzb = ceil_div(g.nz, Job::NP);
     Job job{W, tws, &tmap, bh, g.nz, g.Mxp, g.Ky, g.My, nxb, nzb, nxb * nzb * ncomp, (size_t)X::N * g.Mxp};
@@ -134,7 +135,7 @@ template <class X, bool INV>
 cudaError_t launch(float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st, const CUtensorMap& map,
                    int bh, int* err, cudaStream_t s)
 {
-    constexpr int TX = y_tx<X::N>(), NP = X::C / TX;
+    constexpr int TX = kTX, NP = X::C / TX;
     const long long tiles = (long long)ceil_div(g.Mxp, TX) * ceil_div(g.nz, NP) * ncomp;
     k_ycol<X, INV><<<col_grid<X>(k_ycol<X, INV>, tiles), X::THREADS, X::kSmem, s>>>(W, g, tw, ncomp, st, map, bh, err,
                                                                                     current_batch().mb);

@@ -255,8 +255,10 @@ struct YTile {
 template <typename T> YTile y_tile(const Geom& g, int ncomp)
 {
     YTile t;
-    const int cap = tile_elems<T>();
     const int cmax = g.ycols > 0 ? g.ycols : kThreads;   // columns per tile
+    // 128-byte rows over 512 rows too where the two-pass kernel serves them
+    const bool wide = sizeof(T) == 4 && g.two_pass_y && g.ny > 512 && cmax >= 16 && ycol_serves(g.ny, 16);
+    const int cap = wide ? 2 * tile_elems<T>() : tile_elems<T>();
     int TX = sizeof(T) == 4 ? 16 : 8;                     // 128-byte runs
     while (TX > 1 && (g.ny * TX > cap || TX > cmax)) TX >>= 1;
     int NP = 1;
@@ -345,7 +347,6 @@ cudaError_t launch_y(bool inverse, void* W, const Geom& g, const FftPlan& plan, 
         return cudaGetLastError();
     }
     YTile t = y_tile<T>(g, ncomp);
-    if ((size_t)g.ny << (t.lgTX + t.lgNP) > (size_t)tile_elems<T>()) return cudaErrorInvalidValue;
     cplx<T>* w = (cplx<T>*)W;
     if constexpr (sizeof(T) == 4) {
         if (plan.two_pass && ycol_serves(g.ny, 1 << (t.lgTX + t.lgNP))) {
@@ -354,6 +355,7 @@ cudaError_t launch_y(bool inverse, void* W, const Geom& g, const FftPlan& plan, 
             return launch_ycol(inverse, w, g, tw, ncomp, st, bh > 0 ? (inverse ? maps->inv : maps->fwd) : none, bh, err, s);
         }
     }
+    if ((size_t)g.ny << (t.lgTX + t.lgNP) > (size_t)tile_elems<T>()) return cudaErrorInvalidValue;
     return plan_has_radix16(plan) ? launch_y2<T, true>(inverse, w, g, plan, tw, pos, ncomp, st, maps, err, t, s)
                                   : launch_y2<T, false>(inverse, w, g, plan, tw, pos, ncomp, st, maps, err, t, s);
 }
@@ -384,7 +386,9 @@ template <typename T> cudaError_t prepare_y(void* W, const Geom& g, YMaps* m)
     // every box destination (row offsets of the tile) on a 128-byte boundary
     const size_t row_bytes = sizeof(cplx<T>) << (t.lgTX + t.lgNP);
     m->inv_bh = make(&m->inv, inverse_box_rows(g.ny, g.Ky, row_bytes));
-    m->fwd_bh = make(&m->fwd, forward_box_rows(g.ny, row_bytes));
+    // (a wide tile of a long transform arrives in two halves)
+    const bool halves = sizeof(T) == 4 && g.ny > 512 && (1 << (t.lgTX + t.lgNP)) == 16;
+    m->fwd_bh = make(&m->fwd, forward_box_rows(halves ? g.ny / 2 : g.ny, row_bytes));
     return cudaSuccess;
 }
 

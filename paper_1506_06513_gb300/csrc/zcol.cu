@@ -1,5 +1,5 @@
 // z passes in two register passes (colfft.cuh): the FP32 z transforms of zpass.cu
-// at the lengths of FLUSI_COL_SHORT, full tiles.  A tile is C consecutive
+// at the lengths of FLUSI_COL_LENGTHS, full tiles.  A tile is C consecutive
 // columns q = jy Mxp + x.
 //
 // The inverse pass forms u and omega = i k x u from five transforms per column
@@ -46,21 +46,23 @@ template <class X> struct ZForward {
 
     __device__ __forceinline__ int tile_of(int i) const { return (int)(blockIdx.x + i * gridDim.x); }
     __device__ __forceinline__ bool exists(int i) const { return tile_of(i) < ntiles; }
-    __device__ __forceinline__ void issue(int i, float2* buf, unsigned long long* bar) const
+    // rows h N/CH to (h + 1) N/CH of a tile
+    __device__ __forceinline__ void issue(int i, int h, float2* buf, unsigned long long* bar) const
     {
         const int tile = tile_of(i), c = tile / nqb, q0 = (tile - c * nqb) * C;
-        const int nb = N / bh;
-        mbar_expect_tx(bar, (unsigned)(N * C * sizeof(float2)));
-        for (int b = 0; b < nb; ++b) tma_load_3d(buf + b * bh * C, map, 2 * q0, b * bh, c, bar);
+        constexpr int half = N / X::CH;
+        const int nb = half / bh;
+        mbar_expect_tx(bar, (unsigned)(half * C * sizeof(float2)));
+        for (int b = 0; b < nb; ++b) tma_load_3d(buf + b * bh * C, map, 2 * q0, h * half + b * bh, c, bar);
     }
-    __device__ __forceinline__ void copy(int i, float2* buf, int tid) const
+    __device__ __forceinline__ void copy(int i, int h, float2* buf, int tid) const
     {
         const int tile = tile_of(i), c = tile / nqb;
-        constexpr int lanes = C / 2;
+        constexpr int lanes = C / 2, half = N / X::CH;
         const int col = (tid % lanes) * 2, q = (tile - c * nqb) * C + col;
         if (q >= Q) return;   // Q is a multiple of 4
-        const float2* src = W + (size_t)c * N * plane + q;
-        for (int z = tid / lanes; z < N; z += X::T / lanes) cp_async_16(buf + z * C + col, src + (size_t)z * plane);
+        const float2* src = W + ((size_t)c * N + h * half) * plane + q;
+        for (int z = tid / lanes; z < half; z += X::T / lanes) cp_async_16(buf + z * C + col, src + (size_t)z * plane);
     }
     struct Io {
         const ZForward& job;
@@ -87,13 +89,13 @@ template <class X> struct ZForward {
         }
     };
     template <class Refill>
-    __device__ __forceinline__ void work(int i, float2* buf, int tid, int group, Refill refill) const
+    __device__ __forceinline__ void work(int i, const typename X::Tile& t, int tid, int group, Refill refill) const
     {
         const int tile = tile_of(i), c = tile / nqb, q0 = (tile - c * nqb) * C;
-        X::template first<false, false>(buf, tws, tid, Kz, [](float2 v, int) { return v; });
-        group_sync(group);
+        X::template first<false, false>(t, tws, tid, Kz, [](float2 v, int) { return v; });
+        group_sync<X::T>(group);
         Io io{*this, W + (size_t)c * N * plane, q0, 0, nullptr, false};
-        X::template second<false>(buf, tid, io, refill);
+        X::template second<false>(t, tid, io, refill);
     }
 };
 
@@ -112,7 +114,7 @@ k_zcol_fwd(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, int n
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ ColState state;
     float2* bufs = reinterpret_cast<float2*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
-    float2* tws = bufs + X::BUFS * X::N * X::C;
+    float2* tws = bufs + X::BUFS * X::BUF;
     const int Q = g.My * g.Mxp, nqb = ceil_div(Q, X::C);
     ZForward<X> job{W, tws, &wmap, bh, Q, nqb, nf * nqb, g.Kz, g.Mz, (size_t)g.ny * g.Mxp};
     X::table(tws, tw);
@@ -148,15 +150,17 @@ template <class X> struct ZInverse {
     {
         return phases == 3 ? ph : ph == 0 ? 2 : ph <= 2 ? 0 : 1;
     }
-    __device__ __forceinline__ void issue(int i, float2* buf, unsigned long long* bar) const
+    __device__ __forceinline__ void issue(int i, int h, float2* buf, unsigned long long* bar) const
     {
+        constexpr int CH = X::CH, half = N / CH;
         const int q0 = q0_of(i), ph = phase_of(i), comp = comp_of(ph), kb = (Kz + 1) / bh;
         // the first of two reads of a component keeps its lines in L2
         const unsigned long long pol = phases == 3 ? evict_normal() : ph == 1 || ph == 3 ? evict_last() : evict_first();
-        mbar_expect_tx(bar, (unsigned)(2 * (Kz + 1) * C * sizeof(float2)));
+        mbar_expect_tx(bar, (unsigned)((CH == 1 ? 2 : 1) * (Kz + 1) * C * sizeof(float2)));
         for (int b = 0; b < kb; ++b) {
-            box(buf + b * bh * C, 2 * q0, b * bh, comp, bar, pol);
-            box(buf + (N - Kz - 1 + b * bh) * C, 2 * q0, Kz + b * bh, comp, bar, pol);
+            if (CH == 1 || h == 0) box(buf + b * bh * C, 2 * q0, b * bh, comp, bar, pol);
+            if (CH == 1 || h == 1)
+                box(buf + ((CH == 1 ? N : half) - Kz - 1 + b * bh) * C, 2 * q0, Kz + b * bh, comp, bar, pol);
         }
     }
     __device__ __forceinline__ void box(void* dst, int x, int row, int comp, unsigned long long* bar,
@@ -168,15 +172,15 @@ template <class X> struct ZInverse {
             "l"(map), "r"(x), "r"(row), "r"(comp), "r"(smem_u32(bar)), "l"(pol)
             : "memory");
     }
-    __device__ __forceinline__ void copy(int i, float2* buf, int tid) const
+    __device__ __forceinline__ void copy(int i, int h, float2* buf, int tid) const
     {
-        constexpr int lanes = C / 2;
+        constexpr int lanes = C / 2, half = N / X::CH;
         const int col = (tid % lanes) * 2, q = q0_of(i) + col;
         if (q >= Q) return;   // Q is a multiple of 4
         const float2* src = U + comp_of(phase_of(i)) * ustride + q;
-        for (int s = tid / lanes; s < N; s += X::T / lanes) {
-            const int jz = s <= Kz ? s : (s >= N - Kz ? s - N + Mz : -1);
-            if (jz >= 0) cp_async_16(buf + s * C + col, src + (size_t)jz * Q);
+        for (int o = tid / lanes; o < half; o += X::T / lanes) {
+            const int s = h * half + o, jz = s <= Kz ? s : (s >= N - Kz ? s - N + Mz : -1);
+            if (jz >= 0) cp_async_16(buf + o * C + col, src + (size_t)jz * Q);
         }
     }
     // A transform v of this phase: v itself to out_v (kept in L2 when it is a
@@ -191,8 +195,8 @@ template <class X> struct ZInverse {
         float2 *out_v, *out_c;
         const float2* side;
         unsigned long long pol;
-        static constexpr int H = (L + 1) / 2;
-        float2 a[H];                         // side rows of half the outputs
+        static constexpr int H = L > 18 ? (L + 3) / 4 : (L + 1) / 2;
+        float2 a[H];                         // side rows of the next outputs
 
         __device__ __forceinline__ const float2* side_row(int i) const { return side + (at + (size_t)(R * i) * job.plane); }
         __device__ __forceinline__ float2 side_load(int i) const
@@ -230,9 +234,9 @@ template <class X> struct ZInverse {
             }
 #pragma unroll
             for (int i = 0; i < L; ++i) {
-                if (i == H) {
+                if (i > 0 && i % H == 0) {
 #pragma unroll
-                    for (int u = 0; u < H && H + u < L; ++u) a[u] = side_load(H + u);
+                    for (int u = 0; u < H && i + u < L; ++u) a[u] = side_load(i + u);
                 }
                 const size_t o = at + (size_t)(R * i) * job.plane;
                 const float2 w = a[i % H];
@@ -242,14 +246,14 @@ template <class X> struct ZInverse {
         }
     };
     template <class Refill>
-    __device__ __forceinline__ void work(int i, float2* buf, int tid, int group, Refill refill) const
+    __device__ __forceinline__ void work(int i, const typename X::Tile& t, int tid, int group, Refill refill) const
     {
         const int ph = phase_of(i);
         const bool weighted = phases == 5 && (ph == 1 || ph == 3);
-        X::template first<true, true>(buf, tws, tid, Kz, [&](float2 v, int row) {
+        X::template first<true, true>(t, tws, tid, Kz, [&](float2 v, int row) {
             return weighted ? cscale(v, kzu * float(2 * row <= N ? row : row - N)) : v;
         });
-        group_sync(group);
+        group_sync<X::T>(group);
         Io io{*this, q0_of(i), ph};
         io.pol = phases == 3 ? evict_normal() : ph >= 3 ? evict_first() : evict_last();
         if (phases == 3) {
@@ -261,7 +265,7 @@ template <class X> struct ZInverse {
             io.out_c = ph == 1 ? W + 4 * field : ph == 3 ? W + 3 * field : ph == 4 ? W + 5 * field : nullptr;
             io.side = ph == 1 || ph == 3 ? W + 2 * field : ph == 4 ? W : nullptr;
         }
-        X::template second<true>(buf, tid, io, refill);
+        X::template second<true>(t, tid, io, refill);
     }
 };
 
@@ -282,7 +286,7 @@ k_zcol_inv(const float2* __restrict__ U, float2* __restrict__ W, Geom g, const d
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ ColState state;
     float2* bufs = reinterpret_cast<float2*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
-    float2* tws = bufs + X::BUFS * X::N * X::C;
+    float2* tws = bufs + X::BUFS * X::BUF;
     const int Q = g.My * g.Mxp;
     const float two_pi = 6.283185307179586476925286766559f;
     const size_t plane = (size_t)g.ny * g.Mxp;
@@ -300,7 +304,7 @@ bool zcol_serves(int nz, int cols)
 {
     switch (nz) {
 #define FLUSI_CASE(n, R, L) case n: return cols == z_cols<n>();
-        FLUSI_COL_SHORT(FLUSI_CASE)
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     default: return false;
     }
@@ -318,7 +322,7 @@ cudaError_t launch_zcol_fwd(float2* W, int nf, const Geom& g, const double2* tw,
                                                                                      current_batch().mb);         \
         break;                                                                                                   \
     }
-        FLUSI_COL_SHORT(FLUSI_CASE)
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     default: return cudaErrorInvalidValue;
     }
@@ -337,7 +341,7 @@ cudaError_t launch_zcol_inv(const float2* U, float2* W, const Geom& g, const dou
                                                                                      current_batch().mb);         \
         break;                                                                                                   \
     }
-        FLUSI_COL_SHORT(FLUSI_CASE)
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     default: return cudaErrorInvalidValue;
     }
@@ -353,7 +357,7 @@ cudaError_t configure_zcol()
         if (!e) e = cudaFuncSetAttribute(k_zcol_fwd<X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::kSmem); \
         if (!e) e = cudaFuncSetAttribute(k_zcol_inv<X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::kSmem); \
     }
-    FLUSI_COL_SHORT(FLUSI_CASE)
+    FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     return e;
 }

@@ -635,9 +635,13 @@ template <typename T> int z_tx(const Geom& g, int fields)
 {
     const int cmax = g.zcols > 0 ? g.zcols : 64;   // columns per tile
     int TX = sizeof(T) == 4 ? 16 : 8;
+    const long long tiles = (long long)current_batch().n * fields;
+    // 128-byte rows over 512 rows too where the two-pass kernel serves them
+    if (sizeof(T) == 4 && g.two_pass_z && g.nz > 512 && cmax >= 16 && zcol_serves(g.nz, 16) &&
+        tiles * ceil_div(g.My * g.Mxp, 16) >= kSMs)
+        return 16;
     while (TX > 1 && (g.nz * TX > cap_zi<T>() || TX > cmax)) TX >>= 1;
     while (2 * TX * g.nz <= cap_zi<T>() && 2 * TX <= cmax) TX *= 2;
-    const long long tiles = (long long)current_batch().n * fields;
     while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(g.My * g.Mxp, TX) < kSMs) TX >>= 1;
     return TX;
 }
@@ -650,7 +654,6 @@ cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan
                       cudaStream_t s)
 {
     const int TX = zinv_tx<T>(g);
-    if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0) return cudaErrorInvalidValue;
     const int blocks = ceil_div(g.My * g.Mxp, TX);
     const size_t smem = sizeof(cplx<T>) * ((size_t)g.nz + (size_t)g.nz * TX) + sizeof(rowidx_t) * g.nz + 128;
     const cplx<T>* u = (const cplx<T>*)U;
@@ -666,6 +669,7 @@ cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan
         if (plan.two_pass && zcol_serves(g.nz, TX) && (nf == 3 || nf == 6))
             return launch_zcol_inv(u, w, g, tw, nf, st, m, tma && !B.mb ? bh : 0, err, s);
     }
+    if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0) return cudaErrorInvalidValue;
     const dim3 grid(blocks, 1, B.n);
     if (tma && !B.mb)
         k_zinv<T, true, false><<<grid, kThreadsInv, smem, s>>>(u, w, g, plan, tw, pos, nf, lg, st, m, bh, err, nullptr);
@@ -680,7 +684,7 @@ cudaError_t launch_zf(void* W, int nf, const Geom& g, const FftPlan& plan, const
                       cudaStream_t s)
 {
     const int TX = zfwd_tx<T>(g);
-    if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0 || nf < 1 || nf > 6) return cudaErrorInvalidValue;
+    if (nf < 1 || nf > 6) return cudaErrorInvalidValue;
     const int blocks = nf * ceil_div(g.My * g.Mxp, TX);
     const size_t smem = sizeof(cplx<T>) * ((size_t)g.nz + (size_t)g.nz * TX) + sizeof(rowidx_t) * g.nz + 128;
     cplx<T>* w = (cplx<T>*)W;
@@ -694,6 +698,7 @@ cudaError_t launch_zf(void* W, int nf, const Geom& g, const FftPlan& plan, const
     if constexpr (sizeof(T) == 4) {
         if (plan.two_pass && zcol_serves(g.nz, TX)) return launch_zcol_fwd(w, nf, g, tw, st, m, use_tma ? bh : 0, err, s);
     }
+    if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0) return cudaErrorInvalidValue;
     if (plan_has_radix16(plan)) {
         if (use_tma) k_zfwd<T, true, true><<<grid, kThreadsInv, smem, s>>>(w, g, plan, tw, pos, lg, st, m, bh, err, nullptr);
         else k_zfwd<T, false, true><<<grid, kThreadsInv, smem, s>>>(w, g, plan, tw, pos, lg, st, m, 0, err, B.mb);
@@ -731,7 +736,9 @@ template <typename T> cudaError_t prepare_z(void* U, void* Ut, void* W, const Ge
     const int ibh = inverse_box_rows(g.nz, g.Kz, (size_t)TXi * sizeof(cplx<T>));
     m->u_bh = make(&m->u, U, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
     m->ut_bh = make(&m->ut, Ut, g.Mz, 3, Q, (size_t)g.Mz * Q, ibh, TXi);
-    const int fbh = forward_box_rows(g.nz, (size_t)TXf * sizeof(cplx<T>));
+    // (a wide tile of a long transform arrives in two halves)
+    const bool halves = sizeof(T) == 4 && g.nz > 512 && TXf == 16;
+    const int fbh = forward_box_rows(halves ? g.nz / 2 : g.nz, (size_t)TXf * sizeof(cplx<T>));
     const size_t Wplane = (size_t)g.ny * g.Mxp;
     m->w_bh = make(&m->w, W, g.nz, 6, Wplane, (size_t)g.nz * Wplane, fbh, TXf);
     return cudaSuccess;

@@ -28,7 +28,7 @@ def fl():
 
 def _full(n, most):
     c = 8
-    while 2 * c * n <= 8192 and 2 * c <= most:
+    while 2 * c * n <= (8192 if n <= 512 else 16384) and 2 * c <= most:
         c *= 2
     return c
 
@@ -76,7 +76,7 @@ def test_y_lengths(fl, n):
     _check(fl, (18, n, _smooth_at_least(51 * planes)), cols, 0)
 
 
-@pytest.mark.parametrize("n", [v for v in LENGTHS if v <= 512])
+@pytest.mark.parametrize("n", LENGTHS)
 def test_z_lengths(fl, n):
     cols = _full(n, 64)
     ny = _smooth_at_least(152 * cols * 3 // 2 // 32 + 3)   # My >= 2 ny / 3 - 1 rows of 32 or 36 columns fill 152 tiles
