@@ -72,6 +72,7 @@ template <int R_, int L_, int G_> struct XLine {
     // elements per lane that can be a stored mode (k < Mxp, Mx padded to 4)
     static constexpr int MXP = (2 * NH / 3 + 1 + 3) / 4 * 4;
     static constexpr int NT = (MXP - 1) / L + 1 < R ? (MXP - 1) / L + 1 : R;
+    static constexpr int NA = sq_always<R, L>();           // elements that are kept modes on every lane
 
     static_assert(G * L <= 32, "a warp's lines");
 
@@ -129,14 +130,15 @@ template <int R_, int L_, int G_> struct XLine {
         }
     }
 
-    // Modes -> rows in the slices.  load(k): kept mode k of this lane's line.
-    template <class Load>
+    // Modes -> rows in the slices.  src: this lane's line of Mx kept modes (any
+    // line of the grid where the values are not used).
     __device__ __forceinline__ static void inverse_pass1(float2* slices, const Lane& p, const float2* twx,
-                                                         const float2* tw2, Load load)
+                                                         const float2* tw2, const float2* src, int Mx)
     {
         float2 v[R];
 #pragma unroll
-        for (int t = 0; t < R; ++t) v[t] = t < NT ? load(p.j + L * t) : make_float2(0.0f, 0.0f);
+        for (int t = 0; t < R; ++t)
+            v[t] = t < NA ? src[p.j + L * t] : t < NT && p.j + L * t < Mx ? src[p.j + L * t] : make_float2(0.0f, 0.0f);
         if (p.j == 0) v[0].y = 0.0f;       // a real line has a real mean
         pre(v, p, twx);
         Dft<float, R, true>::run(v);
@@ -177,9 +179,9 @@ template <int R_, int L_, int G_> struct XLine {
         put(s, a);
     }
 
-    // Rows in the slices -> modes.  store(k, X): mode k < MXP of this lane's line.
-    template <class Store>
-    __device__ __forceinline__ static void forward_pass1(const float2* slices, const Lane& p, const float2* twx, Store store)
+    // Rows in the slices -> modes of this lane's line `out` (stored where ok).
+    __device__ __forceinline__ static void forward_pass1(const float2* slices, const Lane& p, const float2* twx, float2* out,
+                                                         bool ok, int Mx, int Mxp)
     {
         float2 v[R];
         const float2* s = slices + p.g * CS + p.j;
@@ -191,7 +193,8 @@ template <int R_, int L_, int G_> struct XLine {
             const float2 o = from(v[R - 1 - q], p.partner);
             const float2 m = p.j != 0 ? o : v[(R - q) % R];
             const int k = p.j + L * q;
-            store(k, v[q], m);
+            const float2 x = q < NA || k < Mx ? r2c_post<float>(v[q], m, twx[k]) : make_float2(0.0f, 0.0f);
+            if (ok && (q < NA || k < Mxp)) out[k] = x;
         }
     }
 
@@ -232,8 +235,7 @@ k_xlines(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XExtra 
         const bool ok = p.on && ln < lines;
         float2* modes = W + ((size_t)ex.comp0 * nrows + (size_t)(ok ? ln : l0)) * Mxp;
         if (MODE != XP_R2C) {
-            X::inverse_pass1(slices, p, twx, tw2,
-                             [&](int k) { return ok && k < Mx ? modes[k] : make_float2(0.0f, 0.0f); });
+            X::inverse_pass1(slices, p, twx, tw2, modes, Mx);
             __syncwarp();
         }
         X::rows(slices, lane, [&](float2* s, int gl, int n1) {
@@ -293,9 +295,7 @@ k_xlines(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XExtra 
         });
         __syncwarp();
         if (MODE != XP_C2R) {
-            X::forward_pass1(slices, p, twx, [&](int k, float2 z, float2 m) {
-                if (ok && k < Mxp) modes[k] = k < Mx ? r2c_post<float>(z, m, twx[k]) : make_float2(0.0f, 0.0f);
-            });
+            X::forward_pass1(slices, p, twx, modes, ok, Mx, Mxp);
             __syncwarp();
         }
     }
@@ -378,8 +378,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                 const bool ok = p.on && r < nrows;
                 const float2* src = W + ((size_t)(cl / RB) * nrows + (ok ? r : 0)) * Mxp;
                 float2* slices = buf + c0 * CS;
-                X::inverse_pass1(slices, p, twx, tw2,
-                                 [&](int k) { return ok && k < Mx ? src[k] : make_float2(0.0f, 0.0f); });
+                X::inverse_pass1(slices, p, twx, tw2, src, Mx);
                 __syncwarp();
                 X::rows(slices, lane, [&](float2* s, int, int) {
                     float2 a[L];
@@ -504,9 +503,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                 });
                 __syncwarp();
                 float2* out = W + ((size_t)(cl / RB) * nrows + (ok ? r : 0)) * Mxp;
-                X::forward_pass1(slices, p, twx, [&](int k, float2 z, float2 m) {
-                    if (ok && k < Mxp) out[k] = k < Mx ? r2c_post<float>(z, m, twx[k]) : make_float2(0.0f, 0.0f);
-                });
+                X::forward_pass1(slices, p, twx, out, ok, Mx, Mxp);
             }
             // no block barrier before the next tile: a warp's next inverse
             // lines are u lines (their readers are behind the barrier above)

@@ -601,6 +601,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
     constexpr int NH = sq_nh<R, S>();
     using Map = SqMap<R, S>;
     constexpr int NT = sq_kept<R, L>();    // line elements per lane that can be kept modes
+    constexpr int NA = sq_always<R, L>();  // those that are on every lane
     constexpr int CS = sq_slice<R, S>();   // line slice (S > 0: logical row R q + j at R q + (j ^ q))
     const int nx = g.nx, Mx = g.Mx, Mxp = g.Mxp;
     const int nrows = g.nz * g.ny;
@@ -689,7 +690,9 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
 #pragma unroll
             for (int t = 0; t < R; ++t) {
                 const int k = j + L * t;
-                if (t < NT) v[t] = (r < nrows && k < Mx) ? src[k] : mkc<T>(0, 0);
+                // (a row outside the grid reads row 0: nothing of it is used)
+                if (t < NA) v[t] = src[k];
+                else if (t < NT) v[t] = k < Mx ? src[k] : mkc<T>(0, 0);
                 else v[t] = mkc<T>(0, 0);   // dropped by the 2/3 rule whatever j is
             }
             if (j == 0) v[0].y = T(0);     // a real line has a real mean
@@ -1011,10 +1014,12 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
                     const int k1 = j + L * q1, k2 = j + L * q2;
                     // Z[nh - k]: the partner's mirror element, lane 0's own
                     const cplx<T> m1 = j != 0 ? b : v[(R - q1) % R];
-                    if (k1 < Mxp) out[k1] = k1 < Mx ? r2c_post<T>(v[q1], m1, twx[k1]) : mkc<T>(0, 0);
+                    if (q1 < NA) out[k1] = r2c_post<T>(v[q1], m1, twx[k1]);
+                    else if (k1 < Mxp) out[k1] = k1 < Mx ? r2c_post<T>(v[q1], m1, twx[k1]) : mkc<T>(0, 0);
                     if (q2 < NT) {
                         const cplx<T> m2 = j != 0 ? a : v[(R - q2) % R];
-                        if (k2 < Mxp) out[k2] = k2 < Mx ? r2c_post<T>(v[q2], m2, twx[k2]) : mkc<T>(0, 0);
+                        if (q2 < NA) out[k2] = r2c_post<T>(v[q2], m2, twx[k2]);
+                        else if (k2 < Mxp) out[k2] = k2 < Mx ? r2c_post<T>(v[q2], m2, twx[k2]) : mkc<T>(0, 0);
                     }
                 }
             }

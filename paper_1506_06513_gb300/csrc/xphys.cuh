@@ -296,6 +296,13 @@ __device__ __forceinline__ cplx<T> c2r_pre_dropped(cplx<T> Xm, cplx<T> wk)
 // Registers t of a lane's line elements k = j + L t, t < R = nh / L, that can
 // hold a mode kept by the 2/3 rule (k <= nx/3 = 2 nh / 3); the others are zero.
 template <int R, int L> constexpr int sq_kept() { return (2 * R * L / 3) / L + 1; }
+// Registers t whose element is a kept mode on every lane, under the strict rule
+// (nx/3 - 1 where 3 divides nx) too: they are loaded and stored without a test.
+template <int R, int L> constexpr int sq_always()
+{
+    const int n = 2 * R * L, modes = (n % 3 == 0 ? n / 3 - 1 : n / 3) + 1;
+    return modes / L;
+}
 
 template <typename T, int R, int L>
 __device__ __forceinline__ void sq_exchange_pre(cplx<T>* x, int j, const cplx<T>* twx)
