@@ -64,18 +64,19 @@ cudaError_t launch_ypass(int fp64, bool inverse, void* W, const Geom& g, const F
                          const double2* tw, const int* pos, int ncomp, const StepState* st,
                          const YMaps* maps, int* err, cudaStream_t s, const FftPlan* half = nullptr,
                          const int* pos_half = nullptr);
-// the two-register-pass y and z kernels (ycol.cu, zcol.cu)
-// a length and tile width served; over 512 rows their tiles have twice the columns
-bool zcol_serves(int nz, int cols);
-cudaError_t launch_zcol_fwd(float2* W, int nf, const Geom& g, const double2* tw, const StepState* st, const CUtensorMap& map,
-                            int bh, int* err, cudaStream_t s);
-cudaError_t launch_zcol_inv(const float2* U, float2* W, const Geom& g, const double2* tw, int nf, const StepState* st,
-                            const CUtensorMap& map, int bh, int* err, cudaStream_t s);
-cudaError_t configure_zcol();
-bool ycol_serves(int ny, int cols);
-cudaError_t launch_ycol(bool inverse, float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st,
+// The two-register-pass y and z kernels (ycol.cu, zcol.cu): the columns of a full
+// tile of a length (0: not served).  y tiles of a full tile's or of 16 columns, z
+// tiles of a full tile's or (up to 512 rows) of 8; the results are the same.
+int ycol_full(int ny);
+cudaError_t launch_ycol(bool inverse, int cols, float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st,
                         const CUtensorMap& map, int bh, int* err, cudaStream_t s);
 cudaError_t configure_ycol();
+int zcol_full(int nz);
+cudaError_t launch_zcol_fwd(int cols, float2* W, int nf, const Geom& g, const double2* tw, const StepState* st,
+                            const CUtensorMap& map, int bh, int* err, cudaStream_t s);
+cudaError_t launch_zcol_inv(int cols, const float2* U, float2* W, const Geom& g, const double2* tw, int nf,
+                            const StepState* st, const CUtensorMap& map, int bh, int* err, cudaStream_t s);
+cudaError_t configure_zcol();
 // 1 when the y passes of this grid take the paired kernel (Geom::ypair)
 int ypass_paired(int fp64, const Geom& g);
 

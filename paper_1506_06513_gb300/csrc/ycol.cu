@@ -1,5 +1,5 @@
 // y passes in two register passes (colfft.cuh): the FP32 y transforms of
-// ypass.cu at the lengths of FLUSI_COL_LENGTHS, full tiles.  A tile is 16
+// ypass.cu at the lengths of FLUSI_COL_LENGTHS.  A tile is 16
 // consecutive x modes of NP consecutive z planes of one component.
 #include "colfft.cuh"
 
@@ -144,26 +144,27 @@ cudaError_t launch(float2* W, const Geom& g, const double2* tw, int ncomp, const
 
 }  // namespace
 
-// Whether the y passes of this grid run here: an FP32 tile of TX x NP columns
-// that is the full tile of a length with a kernel.
-bool ycol_serves(int ny, int cols)
+int ycol_full(int ny)
 {
     switch (ny) {
-#define FLUSI_CASE(n, R, L) case n: return cols == y_cols<n>();
+#define FLUSI_CASE(n, R, L) case n: return y_cols<n>();
         FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
-    default: return false;
+    default: return 0;
     }
 }
 
-cudaError_t launch_ycol(bool inverse, float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st,
+cudaError_t launch_ycol(bool inverse, int cols, float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st,
                         const CUtensorMap& map, int bh, int* err, cudaStream_t s)
 {
     switch (g.ny) {
 #define FLUSI_CASE(n, R, L)                                                                                  \
     case n:                                                                                                  \
-        return inverse ? launch<Col<R, L, y_cols<n>()>, true>(W, g, tw, ncomp, st, map, bh, err, s)           \
-                       : launch<Col<R, L, y_cols<n>()>, false>(W, g, tw, ncomp, st, map, bh, err, s);
+        if (cols == y_cols<n>())                                                                             \
+            return inverse ? launch<Col<R, L, y_cols<n>()>, true>(W, g, tw, ncomp, st, map, bh, err, s)       \
+                           : launch<Col<R, L, y_cols<n>()>, false>(W, g, tw, ncomp, st, map, bh, err, s);     \
+        return inverse ? launch<Col<R, L, kTX>, true>(W, g, tw, ncomp, st, map, bh, err, s)                   \
+                       : launch<Col<R, L, kTX>, false>(W, g, tw, ncomp, st, map, bh, err, s);
         FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     default: return cudaErrorInvalidValue;
@@ -173,13 +174,22 @@ cudaError_t launch_ycol(bool inverse, float2* W, const Geom& g, const double2* t
 cudaError_t configure_ycol()
 {
     cudaError_t e = cudaSuccess;
-#define FLUSI_CASE(n, R, L)                                                                                       \
-    if (!e) e = cudaFuncSetAttribute(k_ycol<Col<R, L, y_cols<n>()>, true>,                                         \
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col<R, L, y_cols<n>()>::kSmem); \
-    if (!e) e = cudaFuncSetAttribute(k_ycol<Col<R, L, y_cols<n>()>, false>,                                        \
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col<R, L, y_cols<n>()>::kSmem);
+    auto one = [&](const void* kernel, size_t smem) {
+        if (!e) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+#define FLUSI_KERNELS(X)                                       \
+    one((const void*)k_ycol<X, true>, X::kSmem);               \
+    one((const void*)k_ycol<X, false>, X::kSmem);
+#define FLUSI_CASE(n, R, L)                                    \
+    {                                                          \
+        using Full = Col<R, L, y_cols<n>()>;                   \
+        using Small = Col<R, L, kTX>;                          \
+        FLUSI_KERNELS(Full)                                    \
+        FLUSI_KERNELS(Small)                                   \
+    }
     FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
+#undef FLUSI_KERNELS
     return e;
 }
 

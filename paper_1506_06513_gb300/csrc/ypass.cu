@@ -252,22 +252,34 @@ struct YTile {
     size_t smem;
 };
 
+// Whether the two-pass kernels run a grid's y passes: by the grid and its tuning
+// alone, whatever the batch, so that members equal solo runs bit for bit.
+template <typename T> bool y_two_pass(const Geom& g)
+{
+    const int full = sizeof(T) == 4 && g.two_pass_y ? ycol_full(g.ny) : 0;
+    return full > 0 && (g.ycols <= 0 || g.ycols >= full);
+}
+
 template <typename T> YTile y_tile(const Geom& g, int ncomp)
 {
     YTile t;
     const int cmax = g.ycols > 0 ? g.ycols : kThreads;   // columns per tile
-    // 128-byte rows over 512 rows too where the two-pass kernel serves them
-    const bool wide = sizeof(T) == 4 && g.two_pass_y && g.ny > 512 && cmax >= 16 && ycol_serves(g.ny, 16);
-    const int cap = wide ? 2 * tile_elems<T>() : tile_elems<T>();
     int TX = sizeof(T) == 4 ? 16 : 8;                     // 128-byte runs
-    while (TX > 1 && (g.ny * TX > cap || TX > cmax)) TX >>= 1;
     int NP = 1;
-    while (2 * NP * TX * g.ny <= cap && 2 * NP * TX <= std::min(kThreads, cmax) && 2 * NP <= g.nz) NP *= 2;
     // small grids: fewer planes per tile until every SM has a block of a
     // three-field pass (rows stay 128 bytes; one tile for every pass of a grid,
     // as its tensor maps are)
     const long long runs = (long long)current_batch().n * ceil_div(g.Mxp, TX) * 3;
-    while (NP > 1 && runs * ceil_div(g.nz, NP) < kSMs) NP >>= 1;
+    if (y_two_pass<T>(g)) {
+        // the two-pass kernel's full tile, or one plane
+        NP = ycol_full(g.ny) / TX;
+        if (NP > g.nz || runs * ceil_div(g.nz, NP) < kSMs) NP = 1;
+    } else {
+        const int cap = tile_elems<T>();
+        while (TX > 1 && (g.ny * TX > cap || TX > cmax)) TX >>= 1;
+        while (2 * NP * TX * g.ny <= cap && 2 * NP * TX <= std::min(kThreads, cmax) && 2 * NP <= g.nz) NP *= 2;
+        while (NP > 1 && runs * ceil_div(g.nz, NP) < kSMs) NP >>= 1;
+    }
     t.lgTX = __builtin_ctz(TX);
     t.lgNP = __builtin_ctz(NP);
     t.blocks = ceil_div(g.Mxp, TX) * ceil_div(g.nz, NP) * ncomp;
@@ -349,10 +361,11 @@ cudaError_t launch_y(bool inverse, void* W, const Geom& g, const FftPlan& plan, 
     YTile t = y_tile<T>(g, ncomp);
     cplx<T>* w = (cplx<T>*)W;
     if constexpr (sizeof(T) == 4) {
-        if (plan.two_pass && ycol_serves(g.ny, 1 << (t.lgTX + t.lgNP))) {
+        const int cols = 1 << (t.lgTX + t.lgNP);
+        if (y_two_pass<T>(g)) {
             const int bh = maps && err && !current_batch().mb ? (inverse ? maps->inv_bh : maps->fwd_bh) : 0;
             const CUtensorMap none{};
-            return launch_ycol(inverse, w, g, tw, ncomp, st, bh > 0 ? (inverse ? maps->inv : maps->fwd) : none, bh, err, s);
+            return launch_ycol(inverse, cols, w, g, tw, ncomp, st, bh > 0 ? (inverse ? maps->inv : maps->fwd) : none, bh, err, s);
         }
     }
     if ((size_t)g.ny << (t.lgTX + t.lgNP) > (size_t)tile_elems<T>()) return cudaErrorInvalidValue;

@@ -1,6 +1,7 @@
 // z passes in two register passes (colfft.cuh): the FP32 z transforms of zpass.cu
-// at the lengths of FLUSI_COL_LENGTHS, full tiles.  A tile is C consecutive
-// columns q = jy Mxp + x.
+// at the lengths of FLUSI_COL_LENGTHS.  A tile is C consecutive columns q = jy Mxp + x:
+// a full tile, or on grids whose full tiles would leave SMs idle 8 (up to 512 rows),
+// with the same arithmetic.
 //
 // The inverse pass forms u and omega = i k x u from five transforms per column
 // range (see k_zinv): W2 = Fz u_z; W4 = i (Fz(kz u_x) - kx W2); W0 = Fz u_x;
@@ -14,6 +15,7 @@ namespace flusi {
 namespace {
 
 template <int N> constexpr int z_cols() { return col_tile(N, 64); }
+constexpr int kZSmall = 8;   // 64-byte rows, which L2 holds on grids that small
 
 __device__ __forceinline__ unsigned long long evict_last()
 {
@@ -299,66 +301,88 @@ k_zcol_inv(const float2* __restrict__ U, float2* __restrict__ W, Geom g, const d
 
 }  // namespace
 
-// Whether the z passes of length nz with tiles of `cols` columns run here.
-bool zcol_serves(int nz, int cols)
+int zcol_full(int nz)
 {
     switch (nz) {
-#define FLUSI_CASE(n, R, L) case n: return cols == z_cols<n>();
+#define FLUSI_CASE(n, R, L) case n: return z_cols<n>();
         FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
-    default: return false;
+    default: return 0;
     }
 }
 
-cudaError_t launch_zcol_fwd(float2* W, int nf, const Geom& g, const double2* tw, const StepState* st, const CUtensorMap& map,
-                            int bh, int* err, cudaStream_t s)
+namespace {
+
+template <class X>
+cudaError_t launch_fwd(float2* W, int nf, const Geom& g, const double2* tw, const StepState* st, const CUtensorMap& map,
+                       int bh, int* err, cudaStream_t s)
 {
-    switch (g.nz) {
-#define FLUSI_CASE(n, R, L)                                                                                      \
-    case n: {                                                                                                    \
-        using X = Col<R, L, z_cols<n>()>;                                                                         \
-        const long long tiles = (long long)nf * ceil_div(g.My * g.Mxp, X::C);                                     \
-        k_zcol_fwd<X><<<col_grid<X>(k_zcol_fwd<X>, tiles), X::THREADS, X::kSmem, s>>>(W, g, tw, nf, st, map, bh, err, \
-                                                                                     current_batch().mb);         \
-        break;                                                                                                   \
-    }
-        FLUSI_COL_LENGTHS(FLUSI_CASE)
-#undef FLUSI_CASE
-    default: return cudaErrorInvalidValue;
-    }
+    const long long tiles = (long long)nf * ceil_div(g.My * g.Mxp, X::C);
+    k_zcol_fwd<X><<<col_grid<X>(k_zcol_fwd<X>, tiles), X::THREADS, X::kSmem, s>>>(W, g, tw, nf, st, map, bh, err,
+                                                                                 current_batch().mb);
     return cudaGetLastError();
 }
+template <class X>
+cudaError_t launch_inv(const float2* U, float2* W, const Geom& g, const double2* tw, int nf, const StepState* st,
+                       const CUtensorMap& map, int bh, int* err, cudaStream_t s)
+{
+    const long long tiles = ceil_div(ceil_div(g.My * g.Mxp, X::C), X::GROUPS);
+    k_zcol_inv<X><<<col_grid<X>(k_zcol_inv<X>, tiles), X::THREADS, X::kSmem, s>>>(U, W, g, tw, nf, st, map, bh, err,
+                                                                                 current_batch().mb);
+    return cudaGetLastError();
+}
+// the small tile of a length that has one
+template <int N> constexpr int z_small() { return N <= 512 ? kZSmall : z_cols<N>(); }
 
-cudaError_t launch_zcol_inv(const float2* U, float2* W, const Geom& g, const double2* tw, int nf, const StepState* st,
+}  // namespace
+
+cudaError_t launch_zcol_fwd(int cols, float2* W, int nf, const Geom& g, const double2* tw, const StepState* st,
                             const CUtensorMap& map, int bh, int* err, cudaStream_t s)
 {
     switch (g.nz) {
-#define FLUSI_CASE(n, R, L)                                                                                      \
-    case n: {                                                                                                    \
-        using X = Col<R, L, z_cols<n>()>;                                                                         \
-        const long long tiles = ceil_div(ceil_div(g.My * g.Mxp, X::C), X::GROUPS);                                \
-        k_zcol_inv<X><<<col_grid<X>(k_zcol_inv<X>, tiles), X::THREADS, X::kSmem, s>>>(U, W, g, tw, nf, st, map, bh, err, \
-                                                                                     current_batch().mb);         \
-        break;                                                                                                   \
-    }
+#define FLUSI_CASE(n, R, L)                                                                                       \
+    case n:                                                                                                       \
+        return cols == z_cols<n>() ? launch_fwd<Col<R, L, z_cols<n>()>>(W, nf, g, tw, st, map, bh, err, s)         \
+                                   : launch_fwd<Col<R, L, z_small<n>()>>(W, nf, g, tw, st, map, bh, err, s);
         FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+}
+
+cudaError_t launch_zcol_inv(int cols, const float2* U, float2* W, const Geom& g, const double2* tw, int nf,
+                            const StepState* st, const CUtensorMap& map, int bh, int* err, cudaStream_t s)
+{
+    switch (g.nz) {
+#define FLUSI_CASE(n, R, L)                                                                                       \
+    case n:                                                                                                       \
+        return cols == z_cols<n>() ? launch_inv<Col<R, L, z_cols<n>()>>(U, W, g, tw, nf, st, map, bh, err, s)      \
+                                   : launch_inv<Col<R, L, z_small<n>()>>(U, W, g, tw, nf, st, map, bh, err, s);
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
+#undef FLUSI_CASE
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t configure_zcol()
 {
     cudaError_t e = cudaSuccess;
-#define FLUSI_CASE(n, R, L)                                                                                     \
-    {                                                                                                           \
-        using X = Col<R, L, z_cols<n>()>;                                                                        \
-        if (!e) e = cudaFuncSetAttribute(k_zcol_fwd<X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::kSmem); \
-        if (!e) e = cudaFuncSetAttribute(k_zcol_inv<X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::kSmem); \
+    auto one = [&](const void* kernel, size_t smem) {
+        if (!e) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+#define FLUSI_KERNELS(X)                                       \
+    one((const void*)k_zcol_fwd<X>, X::kSmem);                 \
+    one((const void*)k_zcol_inv<X>, X::kSmem);
+#define FLUSI_CASE(n, R, L)                                    \
+    {                                                          \
+        using Full = Col<R, L, z_cols<n>()>;                   \
+        using Small = Col<R, L, z_small<n>()>;                 \
+        FLUSI_KERNELS(Full)                                    \
+        FLUSI_KERNELS(Small)                                   \
     }
     FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
+#undef FLUSI_KERNELS
     return e;
 }
 

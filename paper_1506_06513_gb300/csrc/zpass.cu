@@ -625,6 +625,16 @@ k_zupdate(const cplx<T>* __restrict__ Wn, cplx<T>* __restrict__ U, cplx<T>* __re
     }
 }
 
+// Whether the two-pass kernels run a grid's z passes: by the grid and its tuning
+// alone, whatever the batch, so that members equal solo runs bit for bit.  Over 512
+// rows they have one tile, taken where it fills the chip.
+template <typename T> bool z_two_pass(const Geom& g)
+{
+    const int full = sizeof(T) == 4 && g.two_pass_z ? zcol_full(g.nz) : 0;
+    if (full == 0 || (g.zcols > 0 && g.zcols < full)) return false;
+    return g.nz <= 512 || ceil_div(g.My * g.Mxp, full) >= kSMs;
+}
+
 // Columns of a tile: the widest that fits, but on small grids narrower ones
 // (down to 32-byte rows, which L2 holds) until every SM has a block of the pass,
 // which takes `fields` tiles per column range.  The inverse pass handles a
@@ -634,15 +644,16 @@ k_zupdate(const cplx<T>* __restrict__ Wn, cplx<T>* __restrict__ U, cplx<T>* __re
 template <typename T> int z_tx(const Geom& g, int fields)
 {
     const int cmax = g.zcols > 0 ? g.zcols : 64;   // columns per tile
-    int TX = sizeof(T) == 4 ? 16 : 8;
+    const int Q = g.My * g.Mxp;
     const long long tiles = (long long)current_batch().n * fields;
-    // 128-byte rows over 512 rows too where the two-pass kernel serves them
-    if (sizeof(T) == 4 && g.two_pass_z && g.nz > 512 && cmax >= 16 && zcol_serves(g.nz, 16) &&
-        tiles * ceil_div(g.My * g.Mxp, 16) >= kSMs)
-        return 16;
+    if (z_two_pass<T>(g)) {
+        const int full = zcol_full(g.nz);
+        return g.nz > 512 || tiles * ceil_div(Q, full) >= kSMs ? full : 8;
+    }
+    int TX = sizeof(T) == 4 ? 16 : 8;
     while (TX > 1 && (g.nz * TX > cap_zi<T>() || TX > cmax)) TX >>= 1;
     while (2 * TX * g.nz <= cap_zi<T>() && 2 * TX <= cmax) TX *= 2;
-    while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(g.My * g.Mxp, TX) < kSMs) TX >>= 1;
+    while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(Q, TX) < kSMs) TX >>= 1;
     return TX;
 }
 template <typename T> int zinv_tx(const Geom& g) { return z_tx<T>(g, 1); }
@@ -666,8 +677,8 @@ cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan
     if (plan_has_radix16(plan)) return cudaErrorInvalidValue;
     const Batch& B = current_batch();
     if constexpr (sizeof(T) == 4) {
-        if (plan.two_pass && zcol_serves(g.nz, TX) && (nf == 3 || nf == 6))
-            return launch_zcol_inv(u, w, g, tw, nf, st, m, tma && !B.mb ? bh : 0, err, s);
+        if (z_two_pass<T>(g))
+            return launch_zcol_inv(TX, u, w, g, tw, nf, st, m, tma && !B.mb ? bh : 0, err, s);
     }
     if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0) return cudaErrorInvalidValue;
     const dim3 grid(blocks, 1, B.n);
@@ -696,7 +707,7 @@ cudaError_t launch_zf(void* W, int nf, const Geom& g, const FftPlan& plan, const
     const dim3 grid(blocks, 1, B.n);
     const bool use_tma = tma && !B.mb;
     if constexpr (sizeof(T) == 4) {
-        if (plan.two_pass && zcol_serves(g.nz, TX)) return launch_zcol_fwd(w, nf, g, tw, st, m, use_tma ? bh : 0, err, s);
+        if (z_two_pass<T>(g)) return launch_zcol_fwd(TX, w, nf, g, tw, st, m, use_tma ? bh : 0, err, s);
     }
     if (g.nz * TX > cap_zi<T>() || kThreadsInv % TX != 0) return cudaErrorInvalidValue;
     if (plan_has_radix16(plan)) {
