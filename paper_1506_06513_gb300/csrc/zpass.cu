@@ -385,6 +385,62 @@ k_zinv(const cplx<T>* __restrict__ U, cplx<T>* __restrict__ W, Geom g, FftPlan p
     }
 }
 
+// The inverse pass of a small grid, a block per column range and field: the
+// vorticity is formed as the tile is filled, omega_hat = i k x u_hat from the two
+// components it takes, and each of the nf fields has one transform.  The kernel
+// above takes five transforms for six fields, but one after the other in one
+// block: on a grid that cannot fill the chip that chain is the pass's time.
+template <typename T>
+__global__ void __launch_bounds__(kThreadsInv)
+k_zinv_field(const cplx<T>* __restrict__ U, cplx<T>* __restrict__ W, Geom g, FftPlan plan,
+             const double2* __restrict__ tw, const int* __restrict__ pos, int lgTX, const StepState* __restrict__ st,
+             const Member* __restrict__ mb)
+{
+    if (mb) {   // one member of an ensemble batch
+        U = static_cast<const cplx<T>*>(mb[blockIdx.z].U);
+        W = static_cast<cplx<T>*>(mb[blockIdx.z].W);
+        st = mb[blockIdx.z].st;
+    }
+    if (block_leaves(st, nullptr)) return;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int TX = 1 << lgTX;
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
+    cplx<T>* tws = buf + (g.nz << lgTX);
+    rowidx_t* sinv = reinterpret_cast<rowidx_t*>(tws + g.nz);
+    const int Q = g.My * g.Mxp, nz = g.nz, Kz = g.Kz, Mz = g.Mz;
+    const int q0 = blockIdx.x * TX, f = blockIdx.y;
+    const size_t Ustride = (size_t)Mz * Q, Wplane = (size_t)g.ny * g.Mxp;
+    load_tables<T>(tws, nullptr, tw, nullptr, nz, 0);
+    load_inverse_pos(sinv, pos, nz);
+    const T two_pi = T(6.283185307179586476925286766559);
+    // omega_a = i (k_b u_c - k_c u_b), (a, b, c) cyclic
+    const int a = f < 3 ? f : f - 3, b = (a + 1) % 3, c = (a + 2) % 3;
+    for (int i = threadIdx.x; i < (nz << lgTX); i += kThreadsInv) {
+        const int s = i >> lgTX, q = q0 + (i & (TX - 1));
+        const int jz = s <= Kz ? s : (s >= nz - Kz ? s - nz + Mz : -1);
+        cplx<T> v = mkc<T>(0, 0);
+        if (jz >= 0 && q < Q) {
+            const cplx<T>* u = U + (size_t)jz * Q + q;
+            if (f < 3) {
+                v = u[a * Ustride];
+            } else {
+                const int jy = q / g.Mxp, x = q - jy * g.Mxp;
+                const T k[3] = {two_pi * T(x) / T(g.Lx), two_pi * T(mode_of(jy, g.Ky)) / T(g.Ly),
+                                two_pi * T(mode_of(jz, Kz)) / T(g.Lz)};
+                const T kb = b == 0 ? k[0] : b == 1 ? k[1] : k[2], kc = c == 0 ? k[0] : c == 1 ? k[1] : k[2];
+                const cplx<T> ub = u[b * Ustride], uc = u[c * Ustride];
+                v = cmuli(mkc<T>(kb * uc.x - kc * ub.x, kb * uc.y - kc * ub.y));
+            }
+        }
+        buf[i] = v;
+    }
+    __syncthreads();
+    constexpr int V = 2;
+    const int q = q0 + (threadIdx.x % (TX / V)) * V;
+    ZStore<T, V> out{W + (size_t)f * nz * Wplane + (q < Q ? q : 0), Wplane, q < Q};
+    fft_dif_out<T, true, V, false, false>(buf, TX, TX, plan, tws, sinv, out);
+}
+
 // Forward z transform of one component of a column tile: TX consecutive
 // columns q of W[c] (A form, all nz rows) in by 16-byte asynchronous copies,
 // the kept modes jz (2/3 rule) back into rows jz < Mz of the same columns
@@ -659,6 +715,29 @@ template <typename T> int z_tx(const Geom& g, int fields)
 template <typename T> int zinv_tx(const Geom& g) { return z_tx<T>(g, 1); }
 template <typename T> int zfwd_tx(const Geom& g) { return z_tx<T>(g, 3); }
 
+// Whether the inverse pass takes a block per field: under 2^14 values of kept
+// columns, in FP64 2^15, whatever the batch (the two forms round differently and
+// members equal solo runs bit for bit).  A batch fills the chip, where the sixth
+// transform shows, so the line lies where 16 members are about even.  Steps in us
+// with the chain and so, of 1, 4 and 16 members: FP32 32^3 49 47, 56 52, 83 81;
+// 48^3 64 55, 77 73, 167 175; 64^3 62 62, 110 107, 257 283.  FP64 32^3 136 103,
+// 260 201, 595 609; 48^3 259 209, 449 443, 1464 1515; 64^3 321 244, 719 753,
+// 2162 2515.
+template <typename T> bool z_by_field(const Geom& g)
+{
+    return (long long)g.My * g.Mxp * g.nz < (sizeof(T) == 4 ? 1 << 14 : 1 << 15);
+}
+
+// the tile of that kernel: a staged one, as wide as leaves every SM a block
+template <typename T> int zfield_tx(const Geom& g, int nf)
+{
+    int TX = sizeof(T) == 4 ? 16 : 8;
+    while (TX > 2 && (g.nz * TX > cap_zi<T>() ||
+                      (long long)current_batch().n * nf * ceil_div(g.My * g.Mxp, TX) < kSMs))
+        TX >>= 1;
+    return TX;
+}
+
 template <typename T>
 cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan, const double2* tw,
                       const int* pos, int nf, const StepState* st, const CUtensorMap* map, int bh, int* err,
@@ -676,6 +755,14 @@ cudaError_t launch_zi(const void* U, void* W, const Geom& g, const FftPlan& plan
     // the inverse z pass is built without radix-16 stages (its plan has none)
     if (plan_has_radix16(plan)) return cudaErrorInvalidValue;
     const Batch& B = current_batch();
+    // small grids: a block per field (see z_by_field)
+    if (z_by_field<T>(g)) {
+        const int TXf = zfield_tx<T>(g, nf);
+        const size_t need = sizeof(cplx<T>) * ((size_t)g.nz + (size_t)g.nz * TXf) + sizeof(rowidx_t) * g.nz + 128;
+        k_zinv_field<T><<<dim3(ceil_div(g.My * g.Mxp, TXf), nf, B.n), kThreadsInv, need, s>>>(
+            u, w, g, plan, tw, pos, __builtin_ctz(TXf), st, B.mb);
+        return cudaGetLastError();
+    }
     if constexpr (sizeof(T) == 4) {
         if (z_two_pass<T>(g))
             return launch_zcol_inv(TX, u, w, g, tw, nf, st, m, tma && !B.mb ? bh : 0, err, s);
@@ -884,6 +971,8 @@ cudaError_t configure_zpass()
     FLUSI_SMEM_Z(float, true)
     FLUSI_SMEM_Z(double, true)
 #undef FLUSI_SMEM_Z
+    FLUSI_SMEM((k_zinv_field<float>))
+    FLUSI_SMEM((k_zinv_field<double>))
     FLUSI_SMEM((k_zinv<float, false, false>))
     FLUSI_SMEM((k_zinv<float, true, false>))
     FLUSI_SMEM((k_zinv<double, false, false>))

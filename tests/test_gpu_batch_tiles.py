@@ -2,11 +2,13 @@
 run takes narrower y and z tiles than the batch (csrc/ypass.cu, zpass.cu): at
 every length of the two-pass kernels up to 512, and in FP64.  The narrow tiles
 themselves against the FP64 solver (3e-5 after two steps, the bar of the other
-FP32 step tests).
+FP32 step tests), and the inverse z pass by fields (grids under 2^14 values of
+kept columns, FP64 2^15) against the oracle on both sides of those lines.
 """
 import numpy as np
 import pytest
 
+import oracle
 from parity import check_state
 import workloads
 
@@ -77,3 +79,19 @@ def test_z_lengths_in_a_batch(fl, n):
 @pytest.mark.parametrize("n", [(32, 32, 32), (48, 36, 24), (64, 64, 64)])
 def test_fp64_in_a_batch(fl, n):
     _check_batch(fl, n, 6, "fp64")
+
+
+# 0.01, 0.18, 0.88, 0.97 | 1.09, 1.93 | 2.17, 2.5, 4.0 of 2^14; ragged tiles
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [(8, 8, 8), (18, 9, 54), (36, 36, 36), (48, 48, 24), (48, 48, 27), (48, 48, 48),
+                               (48, 54, 48), (12, 8, 1024), (64, 64, 64)])
+def test_inverse_z_by_fields(fl, n, prec):
+    cfg, ins = _case(n)
+    u0 = workloads.random_smooth_field(n, 7, mean=(0.3, 0.0, 0.0))
+    u, rows = _solo(fl, cfg, ins, u0, prec)
+    ref = oracle.Simulation(cfg, ins)
+    ref.set_state(u0)
+    want = ref.step(2)
+    tol, tol_rows = (1e-11, 1e-10) if prec == "fp64" else (3e-5, 1e-4)
+    check_state(u, ref.get_state(), tol)
+    assert np.linalg.norm(rows[:, 2:22] - want[:, 2:22]) <= tol_rows * np.linalg.norm(want[:, 2:22])
