@@ -483,7 +483,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                                 cross3(rv, pu, acc + 3);
                                 cross3(rv, cu, acc + 9);
                             }
-                            warp_sums12<float>(acc, wacc + warp * 36 + cc * 12, lane);
+                            warp_sums12(acc, wacc + warp * 36 + cc * 12, lane);
                         }
                     }
                 }

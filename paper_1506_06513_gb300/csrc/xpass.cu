@@ -427,7 +427,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
                             }
                         }
                         // a lane's points in T, everything above it in FP64
-                        warp_sums12<T>(v, wacc + warp * 36 + cc * 12, lane);
+                        warp_sums12(v, wacc + warp * 36 + cc * 12, lane);
                     }
                 }
             }
@@ -924,7 +924,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
                         }
                         // one point per lane in T; the sums across lanes, warps
                         // and blocks in FP64
-                        warp_sums12<T>(acc, wacc + warp * 36 + cc * 12, lane);
+                        warp_sums12(acc, wacc + warp * 36 + cc * 12, lane);
                     }
                 }
             }

@@ -230,20 +230,61 @@ __device__ __forceinline__ double warp_sum(double v)
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// c2r pre-processing: Z[k] = (X[k] + X*[m]) + i (X[k] - X*[m]) w^{-k} with the
-// mirror value Xm = X[nh - k].
-// The warp totals of 12 per-lane values in FP64, added into w[0..11]: a
-// reduce-scatter over 16 slots (12 values, 4 zeros), halving the slots per
-// lane at each of the xor-16, 8, 4, 2 exchanges, then one xor-1 add; lane
-// 2i + 1 (bits 4..1 = i) ends with the total of slot i.  16 FP64 adds a warp
-// instead of the 60 of twelve separate butterflies (FP64 is slow here).
-// Every lane of the warp calls it.
-template <typename T>
-__device__ __forceinline__ void warp_sums12(const T* v, double* w, int lane)
+// hi + lo + x without a rounding in FP32 but that of lo (two-sum; Knuth, TAOCP 4.2.2)
+__device__ __forceinline__ void two_add(float& hi, float& lo, float x)
+{
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
+}
+
+// The warp totals of 12 per-lane values, added into w[0..11]: a reduce-scatter
+// over 16 slots (12 values, 4 zeros), halving the slots per lane at each of the
+// xor-16, 8, 4, 2 exchanges, then one xor-1 add; lane 2i + 1 (bits 4..1 = i) ends
+// with the total of slot i.  Every lane of the warp calls it.
+//
+// FP64 issues one warp instruction in some 17 cycles of an SM: with FP64 sums (12
+// conversions and 16 adds per warp) they, not the line transforms, set the time of
+// tiles with penalized points.  FP32 values are therefore summed over the warp as
+// pairs hi + lo (48 bits) in FP32 instructions, and FP64 above it: x pass with a
+// sphere of 0.3 box lengths at 256^3 286 -> 232 us (158 without a body), at 162^3
+// 102 -> 78, 48 x 36 x 24 with an insect 22 -> 18.  Sums kept per lane over a tile
+// cost registers that the transforms need: 512^3 x pass 1090 -> 1171 us.
+__device__ __forceinline__ void warp_sums12(const float* v, double* w, int lane)
+{
+    float h[8], l[8];
+    const bool up16 = (lane & 16) != 0;   // this lane keeps the upper half
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float top = k < 4 ? v[k + 8] : 0.0f;
+        const float x = __shfl_xor_sync(0xffffffffu, up16 ? v[k] : top, 16);
+        h[k] = up16 ? top : v[k];
+        l[k] = 0.0f;
+        two_add(h[k], l[k], x);
+    }
+#pragma unroll
+    for (int n = 4; n >= 1; n >>= 1) {
+        const bool up = (lane & (2 * n)) != 0;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const float xh = __shfl_xor_sync(0xffffffffu, up ? h[k] : h[k + n], 2 * n);
+            const float xl = __shfl_xor_sync(0xffffffffu, up ? l[k] : l[k + n], 2 * n);
+            h[k] = up ? h[k + n] : h[k];
+            l[k] = __fadd_rn(up ? l[k + n] : l[k], xl);
+            two_add(h[k], l[k], xh);
+        }
+    }
+    const float xh = __shfl_xor_sync(0xffffffffu, h[0], 1), xl = __shfl_xor_sync(0xffffffffu, l[0], 1);
+    l[0] = __fadd_rn(l[0], xl);
+    two_add(h[0], l[0], xh);
+    const int slot = (lane >> 1) & 15;
+    if ((lane & 1) && slot < 12) w[slot] += double(h[0]) + double(l[0]);
+}
+__device__ __forceinline__ void warp_sums12(const double* v, double* w, int lane)
 {
     double d[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) d[k] = k < 12 ? double(v[k]) : 0.0;
+    for (int k = 0; k < 16; ++k) d[k] = k < 12 ? v[k] : 0.0;
 #pragma unroll
     for (int h = 8; h >= 1; h >>= 1) {
         const bool up = (lane & (2 * h)) != 0;   // this lane keeps the upper half
@@ -259,6 +300,8 @@ __device__ __forceinline__ void warp_sums12(const T* v, double* w, int lane)
     if ((lane & 1) && slot < 12) w[slot] += d[0];
 }
 
+// c2r pre-processing: Z[k] = (X[k] + X*[m]) + i (X[k] - X*[m]) w^{-k} with the
+// mirror value Xm = X[nh - k].
 template <typename T>
 __device__ __forceinline__ cplx<T> c2r_pre(cplx<T> Xk, cplx<T> Xm, cplx<T> wk)
 {
