@@ -426,7 +426,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
                                 }
                             }
                         }
-                        // a lane's points in T, everything above it in FP64
+                        // a lane's points in T, everything above the warp in FP64
                         warp_sums12(v, wacc + warp * 36 + cc * 12, lane);
                     }
                 }
@@ -922,8 +922,8 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
                                 acc[9 + q] = m2[q];
                             }
                         }
-                        // one point per lane in T; the sums across lanes, warps
-                        // and blocks in FP64
+                        // one point per lane in T; the sums across warps and
+                        // blocks in FP64
                         warp_sums12(acc, wacc + warp * 36 + cc * 12, lane);
                     }
                 }
@@ -1072,6 +1072,10 @@ template <typename T, int R, int S> size_t sq_smem(const Geom& g, bool sponge = 
     return s;
 }
 
+// Whether lines without the sponge run here: in FP32 not those of 256, 128 and 64
+// points (phys_line).
+template <typename T, int R> constexpr bool sq_plain() { return sizeof(T) == 8 || R != 8; }
+
 // grid = the virtual CTAs (rows of partial sums, x_grid, whichever kernel it was
 // counted for); a batch of n members runs about one resident wave in all, each CTA taking several
 // virtual ones, instead of n full grids of CTAs that each take one or two
@@ -1089,19 +1093,21 @@ void launch_sq(bool layer, bool sponge, cplx<T>* w, const Geom& g, const double2
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, false>, 192, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, !sq_plain<T, R>()>, 192, smem);
         const int resident = std::max(1, sms * std::max(1, per_sm));
         run = std::min(grid, std::max(1, ceil_div(resident, B.n)));
     }
     const dim3 gd(run, 1, B.n);
-    if (layer && sponge)
+    if (layer && sponge) {
         k_xpass_sq<T, R, S, true, true><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
-    else if (layer)
-        k_xpass_sq<T, R, S, true, false><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
-    else if (sponge)
+    } else if (sponge) {
         k_xpass_sq<T, R, S, false, true><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
-    else
-        k_xpass_sq<T, R, S, false, false><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
+    } else if constexpr (sq_plain<T, R>()) {
+        if (layer)
+            k_xpass_sq<T, R, S, true, false><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
+        else
+            k_xpass_sq<T, R, S, false, false><<<gd, 192, smem, s>>>(w, g, tw, ex, st, B.mb);
+    }
 }
 
 // the register-resident kernel for this grid: 10 R + S (R = 16 or 8 with
@@ -1160,7 +1166,7 @@ template <typename T> int x_grid(const Geom& g)
     const XLineOps* line = phys_line<T>(g, false);
 #define FLUSI_SQ_OCC(R, S)                                                                          \
     ntiles = ceil_div(g.nz * g.ny, sq_rows<sq_lanes<R, S>()>());                                               \
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, false>, 192, \
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, !sq_plain<T, R>()>, 192, \
                                                   sq_smem<T, R, S>(g));
     if (line) {
         ntiles = ceil_div(g.nz * g.ny, line->rows);
@@ -1304,8 +1310,10 @@ cudaError_t configure_xpass()
     FLUSI_SMEM((k_xpass<double, XP_C2R>))
     FLUSI_SMEM((k_xpass<double, XP_DUMP>))
 #define FLUSI_SMEM_SQ(T, R, S)                              \
-    FLUSI_SMEM((k_xpass_sq<T, R, S, false, false>))         \
-    FLUSI_SMEM((k_xpass_sq<T, R, S, true, false>))          \
+    if constexpr (sq_plain<T, R>()) {                       \
+        FLUSI_SMEM((k_xpass_sq<T, R, S, false, false>))     \
+        FLUSI_SMEM((k_xpass_sq<T, R, S, true, false>))      \
+    }                                                       \
     FLUSI_SMEM((k_xpass_sq<T, R, S, false, true>))          \
     FLUSI_SMEM((k_xpass_sq<T, R, S, true, true>))
     FLUSI_SMEM_SQ(float, 16, 1)

@@ -732,7 +732,7 @@ template <typename T> bool z_by_field(const Geom& g)
 template <typename T> int zfield_tx(const Geom& g, int nf)
 {
     int TX = sizeof(T) == 4 ? 16 : 8;
-    while (TX > 2 && (g.nz * TX > cap_zi<T>() ||
+    while (TX > 2 && (g.nz * TX > cap_zi<T>() || (g.zcols > 0 && TX > g.zcols) ||
                       (long long)current_batch().n * nf * ceil_div(g.My * g.Mxp, TX) < kSMs))
         TX >>= 1;
     return TX;

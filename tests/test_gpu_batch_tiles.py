@@ -81,10 +81,11 @@ def test_fp64_in_a_batch(fl, n):
     _check_batch(fl, n, 6, "fp64")
 
 
-# 0.01, 0.18, 0.88, 0.97 | 1.09, 1.93 | 2.17, 2.5, 4.0 of 2^14; ragged tiles
+# 0.01, 0.18, 0.79, 0.88, 0.97 | 1.09, 1.25, 1.93 | 2.17, 2.5, 4.0 of 2^14; ragged tiles,
+# lengths that narrow them
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
-@pytest.mark.parametrize("n", [(8, 8, 8), (18, 9, 54), (36, 36, 36), (48, 48, 24), (48, 48, 27), (48, 48, 48),
-                               (48, 54, 48), (12, 8, 1024), (64, 64, 64)])
+@pytest.mark.parametrize("n", [(8, 8, 8), (18, 9, 54), (8, 8, 648), (36, 36, 36), (48, 48, 24), (48, 48, 27), (8, 8, 1024),
+                               (48, 48, 48), (48, 54, 48), (12, 8, 1024), (64, 64, 64)])
 def test_inverse_z_by_fields(fl, n, prec):
     cfg, ins = _case(n)
     u0 = workloads.random_smooth_field(n, 7, mean=(0.3, 0.0, 0.0))
