@@ -344,6 +344,8 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * whose widest tiles would not fill the GPU, a narrower one), else a cap on the tile's columns (x columns times z planes
  * for y; columns of the flattened (y, x) plane for z), a power of two of at
  * least 32 bytes of complex values (4 in FP32, 2 in FP64) and at most 256.
+ * Grids under 2^14 values of kept columns (My Mxp nz; FP64 2^15) take their
+ * inverse z pass a block per column range and field, whatever the plan.
  * x_kernel: 0 (default) the register-resident line kernel where one exists
  * (nx = 128, 256, 512, 1024, and its rectangular form at nx = 64, 96; in FP32
  * the general line kernels at every other length from 16 on), 1 the
