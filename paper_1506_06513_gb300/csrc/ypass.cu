@@ -266,10 +266,13 @@ template <typename T> YTile y_tile(const Geom& g, int ncomp)
     const int cmax = g.ycols > 0 ? g.ycols : kThreads;   // columns per tile
     int TX = sizeof(T) == 4 ? 16 : 8;                     // 128-byte runs
     int NP = 1;
-    // small grids: fewer planes per tile until every SM has a block of a
-    // three-field pass (rows stay 128 bytes; one tile for every pass of a grid,
-    // as its tensor maps are)
-    const long long runs = (long long)current_batch().n * ceil_div(g.Mxp, TX) * 3;
+    // small grids: fewer planes per tile until every SM has a block of the
+    // six-field pass (rows stay 128 bytes; one tile for every pass of a grid, as
+    // its tensor maps are).  Not further: with a block per SM for three fields the
+    // inverse pass took two waves of the two FP64 blocks that an SM holds (inverse
+    // y 32^3 FP64 23 us against 14, step of 48^3 196 and 172, FP32 60 and 54; 96 x
+    // 48 x 64 388 and 351, 61 and 55)
+    const long long runs = (long long)current_batch().n * ceil_div(g.Mxp, TX) * 6;
     if (y_two_pass<T>(g)) {
         // the two-pass kernel's full tile, or one plane
         NP = ycol_full(g.ny) / TX;

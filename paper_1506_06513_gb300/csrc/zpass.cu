@@ -696,7 +696,9 @@ template <typename T> bool z_two_pass(const Geom& g)
 // which takes `fields` tiles per column range.  The inverse pass handles a
 // column range in one block, a serial chain of five transforms (zinv at 128^3
 // FP32: 59 tiles of 64 columns 35 us, 234 of 16 24 us; at 32^3 FP64 4 tiles
-// 67 us, 126 of 2 columns 52 us); the forward pass has a block per field.
+// 67 us, 126 of 2 columns 52 us); the forward pass has a block per field, and
+// narrows as if it had six (with three, 249 blocks of 48^3 FP64 were two waves:
+// 33 us, 126 blocks 18).
 template <typename T> int z_tx(const Geom& g, int fields)
 {
     const int cmax = g.zcols > 0 ? g.zcols : 64;   // columns per tile
@@ -713,7 +715,7 @@ template <typename T> int z_tx(const Geom& g, int fields)
     return TX;
 }
 template <typename T> int zinv_tx(const Geom& g) { return z_tx<T>(g, 1); }
-template <typename T> int zfwd_tx(const Geom& g) { return z_tx<T>(g, 3); }
+template <typename T> int zfwd_tx(const Geom& g) { return z_tx<T>(g, 6); }
 
 // Whether the inverse pass takes a block per field: under 2^14 values of kept
 // columns, in FP64 2^15, whatever the batch (the two forms round differently and

@@ -68,12 +68,17 @@ def _check_batch(fl, n, count, prec):
 
 @pytest.mark.parametrize("n", LENGTHS)
 def test_y_lengths_in_a_batch(fl, n):
-    _check_batch(fl, (18, n, 48), 10, "fp32")   # 3 and 30 runs of 48 planes, by 1 and by up to 8
+    _check_batch(fl, (18, n, 48), 10, "fp32")   # 6 and 60 runs of 48 planes, by 1 and by up to 8
 
 
 @pytest.mark.parametrize("n", LENGTHS)
 def test_z_lengths_in_a_batch(fl, n):
     _check_batch(fl, (96, 96, n), 5, "fp32")    # 37 to 147 and 185 to 735 full tiles
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_z_forward_lengths_in_a_batch(fl, n):
+    _check_batch(fl, (24, 24, n), 10, "fp32")   # 24 to 78 and 240 to 780 full tiles of six fields
 
 
 @pytest.mark.parametrize("n", [(32, 32, 32), (48, 36, 24), (64, 64, 64)])
