@@ -55,9 +55,12 @@ template <int R_, int L_, int C_> struct Col {
     static constexpr bool SMALL = R <= 18 && L <= 18;
     static constexpr int GROUPS = SMALL || CH == 2 ? 1 : 2, BUFS = SMALL ? 1 : 3;
     static constexpr int THREADS = GROUPS * T, MINB = SMALL ? 3 : 1;
-    static constexpr int BUF = N * C / CH;                     // values of a buffer
+    // values of a buffer: a row range, up to the next 128-byte boundary, where the
+    // next buffer's TMA boxes land (243 rows of 8 columns end 64 bytes short of one)
+    static constexpr int BUF = (N * C / CH + 15) / 16 * 16;
     static constexpr size_t kSmem = sizeof(float2) * ((size_t)BUFS * BUF + N) + 128;
     static_assert((C & (C - 1)) == 0 && BUF <= 8192 && (CH == 1 || (R % 2 == 0 && !SMALL)), "a tile");
+    static_assert(BUFS == 1 || BUF * sizeof(float2) % 128 == 0, "TMA destinations");
 
     // A tile: the buffer of its rows, or of its first and its second half of rows.
     struct Tile {
