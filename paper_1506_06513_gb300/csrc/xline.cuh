@@ -316,7 +316,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (st && st->status != 0) return;
+    if (block_leaves(st, nullptr)) return;
     constexpr int NT = 96, NW = 3;
     constexpr int R = X::R, L = X::L, G = X::G, NH = X::NH, CS = X::CS, LP = X::LP;
     constexpr int RB = G, NG = NW * G;         // rows of a tile, lane groups of the block

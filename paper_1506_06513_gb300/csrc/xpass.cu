@@ -200,7 +200,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (st && st->status != 0) return;
+    if (block_leaves(st, nullptr)) return;
     constexpr bool kPhys = (MODE == XP_PHYS || MODE == XP_DUMP);
     const int RB = 1 << lgRB;
     const int NF = kPhys ? 6 : ex.ncomp;
@@ -595,7 +595,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (st && st->status != 0) return;
+    if (block_leaves(st, nullptr)) return;
     constexpr int L = sq_lanes<R, S>();    // lanes per line
     constexpr int RB = sq_rows<L>();
     constexpr int NH = sq_nh<R, S>();
