@@ -320,6 +320,9 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
     constexpr int NT = 96, NW = 3;
     constexpr int R = X::R, L = X::L, G = X::G, NH = X::NH, CS = X::CS, LP = X::LP;
     constexpr int RB = G, NG = NW * G;         // rows of a tile, lane groups of the block
+    // lengths whose sponge runs in a square kernel (xpass.cu): those refuse a state
+    // whose energy overflows, and so does this one
+    constexpr bool ENERGY = NH == 32 || NH == 64 || NH == 128;
     const int Mx = g.Mx, Mxp = g.Mxp;
     const int nrows = g.nz * g.ny;
     const int ntiles = ceil_div(nrows, RB);
@@ -390,9 +393,10 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
             __syncthreads();
 
             // physical space: NL = u x omega into the omega lines, energy and
-            // max |u|^2, a point pair per thread; a non-finite velocity makes
-            // the energy sum non-finite (see k_xpass_sq)
-            float2 e2 = make_float2(0.0f, 0.0f);
+            // max |u|^2, a point pair per thread.  An NL value that is not finite
+            // turns `odd` into NaN (0 times it).  A u that is not makes the energy
+            // sum so, but a large finite u does too: then the values are looked at.
+            float2 e2 = make_float2(0.0f, 0.0f), odd = make_float2(0.0f, 0.0f);
 #pragma unroll 2
             for (int i = tid; i < RB * NH; i += NT) {
                 const int rr = i / NH, lrow = i - rr * NH;
@@ -421,11 +425,25 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                 e2 = __fadd2_rn(e2, uu);
                 m_acc = fmaxf(m_acc, fmaxf(uu.x, uu.y));
 #pragma unroll
-                for (int q = 0; q < 3; ++q) buf[((3 + q) * RB + rr) * CS + slot] = nl[q];
+                for (int q = 0; q < 3; ++q) {
+                    buf[((3 + q) * RB + rr) * CS + slot] = nl[q];
+                    odd = __ffma2_rn(nl[q], make_float2(0.0f, 0.0f), odd);
+                }
             }
             const float e_tile = e2.x + e2.y;
             e_acc += double(e_tile);
-            if (!isfinite(e_tile)) bad = 1;
+            float odd_tile = odd.x + odd.y;
+            if (!isfinite(e_tile)) {
+                if (ENERGY) bad = 1;
+                for (int i = tid; i < RB * NH; i += NT) {
+                    const int rr = i / NH, lrow = i - rr * NH;
+                    if (row0 + rr >= nrows) continue;
+                    for (int q = 0; q < 3; ++q) {
+                        const float2 u = buf[(q * RB + rr) * CS + lrow / L * LP + lrow % L];
+                        if (!isfinite(u.x) || !isfinite(u.y)) bad = 1;
+                    }
+                }
+            }
 
             // penalization, only in tiles with a row that meets a part's box
             int tile_any = 0;
@@ -459,6 +477,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                                 float* nl = reinterpret_cast<float*>(buf + ((3 + q) * RB + rr) * CS + slot);
                                 u[q] = ul[h];
                                 nl[h] -= pen * (u[q] - us[q]);
+                                odd_tile = __fmaf_rn(nl[h], 0.0f, odd_tile);
                             }
                         }
                     }
@@ -488,6 +507,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                     }
                 }
             }
+            if (!(odd_tile == 0.0f)) bad = 1;
             __syncthreads();
 
             // forward on the three NL lines of each row, one per lane group
