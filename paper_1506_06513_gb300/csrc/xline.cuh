@@ -485,7 +485,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
                         for (int cc = 0; cc < 3; ++cc) {
                             const bool has = colr == cc + 1;
                             if (!__any_sync(0xffffffffu, has)) continue;
-                            float acc[12];   // this lane's point in FP32, everything above the warp in FP64
+                            float acc[12];   // this lane's point in FP32, the sums above in FP64 or closer
 #pragma unroll
                             for (int k2 = 0; k2 < 12; ++k2) acc[k2] = 0.0f;
                             if (has) {

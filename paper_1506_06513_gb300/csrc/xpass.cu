@@ -426,7 +426,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
                                 }
                             }
                         }
-                        // a lane's points in T, everything above the warp in FP64
+                        // a lane's points in T, the sums over lanes and above in FP64 or closer
                         warp_sums12(v, wacc + warp * 36 + cc * 12, lane);
                     }
                 }
@@ -922,8 +922,8 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
                                 acc[9 + q] = m2[q];
                             }
                         }
-                        // one point per lane in T; the sums across warps and
-                        // blocks in FP64
+                        // one point per lane in T; the sums across lanes, warps
+                        // and blocks in FP64 or closer
                         warp_sums12(acc, wacc + warp * 36 + cc * 12, lane);
                     }
                 }

@@ -230,56 +230,38 @@ __device__ __forceinline__ double warp_sum(double v)
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// hi + lo + x without a rounding in FP32 but that of lo (two-sum; Knuth, TAOCP 4.2.2)
-__device__ __forceinline__ void two_add(float& hi, float& lo, float x)
+// a + b rounded, and in e what the rounding dropped (two-sum; Knuth, TAOCP 4.2.2)
+__device__ __forceinline__ float two_sum(float a, float b, float& e)
 {
-    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    hi = s;
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
 }
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& e)
+{
+    const float2 s = cadd(a, b), t = csub(s, a);
+    e = cadd(csub(a, csub(s, t)), csub(b, t));
+    return s;
+}
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return cadd(a, b); }
+// h + l + m += x + y + z, three parts of falling size (V: float, or two sums packed);
+// only the last part is rounded, some 70 bits below the first
+template <class V> __device__ __forceinline__ void triple_add(V& h, V& l, V& m, V x, V y, V z)
+{
+    V e1, e2, e3;
+    h = two_sum(h, x, e1);
+    l = two_sum(l, y, e2);
+    l = two_sum(l, e1, e3);
+    m = add(add(m, z), add(e2, e3));
+}
+__device__ __forceinline__ float lane_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float2 lane_xor(float2 v, int o) { return make_float2(lane_xor(v.x, o), lane_xor(v.y, o)); }
 
-// The warp totals of 12 per-lane values, added into w[0..11]: a reduce-scatter
-// over 16 slots (12 values, 4 zeros), halving the slots per lane at each of the
-// xor-16, 8, 4, 2 exchanges, then one xor-1 add; lane 2i + 1 (bits 4..1 = i) ends
-// with the total of slot i.  Every lane of the warp calls it.
-//
-// FP64 issues one warp instruction in some 17 cycles of an SM: with FP64 sums (12
-// conversions and 16 adds per warp) they, not the line transforms, set the time of
-// tiles with penalized points.  FP32 values are therefore summed over the warp as
-// pairs hi + lo (48 bits) in FP32 instructions, and FP64 above it: x pass with a
-// sphere of 0.3 box lengths at 256^3 286 -> 232 us (158 without a body), at 162^3
-// 102 -> 78, 48 x 36 x 24 with an insect 22 -> 18.  Sums kept per lane over a tile
-// cost registers that the transforms need: 512^3 x pass 1090 -> 1171 us.
-__device__ __forceinline__ void warp_sums12(const float* v, double* w, int lane)
-{
-    float h[8], l[8];
-    const bool up16 = (lane & 16) != 0;   // this lane keeps the upper half
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const float top = k < 4 ? v[k + 8] : 0.0f;
-        const float x = __shfl_xor_sync(0xffffffffu, up16 ? v[k] : top, 16);
-        h[k] = up16 ? top : v[k];
-        l[k] = 0.0f;
-        two_add(h[k], l[k], x);
-    }
-#pragma unroll
-    for (int n = 4; n >= 1; n >>= 1) {
-        const bool up = (lane & (2 * n)) != 0;
-#pragma unroll
-        for (int k = 0; k < n; ++k) {
-            const float xh = __shfl_xor_sync(0xffffffffu, up ? h[k] : h[k + n], 2 * n);
-            const float xl = __shfl_xor_sync(0xffffffffu, up ? l[k] : l[k + n], 2 * n);
-            h[k] = up ? h[k + n] : h[k];
-            l[k] = __fadd_rn(up ? l[k + n] : l[k], xl);
-            two_add(h[k], l[k], xh);
-        }
-    }
-    const float xh = __shfl_xor_sync(0xffffffffu, h[0], 1), xl = __shfl_xor_sync(0xffffffffu, l[0], 1);
-    l[0] = __fadd_rn(l[0], xl);
-    two_add(h[0], l[0], xh);
-    const int slot = (lane >> 1) & 15;
-    if ((lane & 1) && slot < 12) w[slot] += double(h[0]) + double(l[0]);
-}
+// The warp totals of 12 per-lane values in FP64, added into w[0..11]: a
+// reduce-scatter over 16 slots (12 values, 4 zeros), halving the slots per lane at
+// each of the xor-16, 8, 4, 2 exchanges, then one xor-1 add; lane 2i + 1 (bits 4..1
+// = i) ends with the total of slot i.  Every lane of the warp calls it.
 __device__ __forceinline__ void warp_sums12(const double* v, double* w, int lane)
 {
     double d[16];
@@ -290,14 +272,70 @@ __device__ __forceinline__ void warp_sums12(const double* v, double* w, int lane
         const bool up = (lane & (2 * h)) != 0;   // this lane keeps the upper half
 #pragma unroll
         for (int k = 0; k < h; ++k) {
-            const double send = up ? d[k] : d[k + h];
             const double keep = up ? d[k + h] : d[k];
+            const double send = up ? d[k] : d[k + h];
             d[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
         }
     }
     d[0] += __shfl_xor_sync(0xffffffffu, d[0], 1);
     const int slot = (lane >> 1) & 15;
     if ((lane & 1) && slot < 12) w[slot] += d[0];
+}
+
+// The same for FP32 values, with no more error: FP64 issues one warp instruction in
+// some 17 cycles of an SM, and with FP64 sums (12 conversions and 16 adds per warp)
+// they, not the line transforms, set the time of tiles with penalized points.  The
+// tree therefore runs in FP32 instructions on values of three parts, of which only
+// what lies some 70 bits below the largest is ever rounded; FP64 adds the parts and
+// everything above the warp.  x pass with a sphere of 0.3 box lengths at 256^3: FP64
+// tree 286 us, this one 245 (156 without a body; with two parts, 48 bits, 232).  Sums
+// kept per lane over a tile cost registers that the transforms need: 512^3 x pass
+// 1090 -> 1171 us.  Where a partial sum could leave the FP32 range, and
+// for infinities and NaN, the warp takes the FP64 tree.
+__device__ __forceinline__ void warp_sums12(const float* v, double* w, int lane)
+{
+    float size = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) size = __fadd_rn(size, fabsf(v[k]));
+    if (__any_sync(0xffffffffu, !(size < 0x1p120f))) {   // 32 lanes of less stay under 2^125
+        double d[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) d[k] = double(v[k]);
+        warp_sums12(d, w, lane);
+        return;
+    }
+    // pairs of neighbouring slots
+    float2 h[4], l[4], m[2];
+    const bool up16 = (lane & 16) != 0;   // this lane keeps the upper half
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 low = make_float2(v[2 * k], v[2 * k + 1]);
+        const float2 top = k < 2 ? make_float2(v[2 * k + 8], v[2 * k + 9]) : make_float2(0.0f, 0.0f);
+        h[k] = two_sum(up16 ? top : low, lane_xor(up16 ? low : top, 16), l[k]);   // two parts hold it
+    }
+#pragma unroll
+    for (int n = 2; n >= 1; n >>= 1) {
+        const bool up = (lane & (4 * n)) != 0;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            if (n == 2) m[k] = make_float2(0.0f, 0.0f);
+            const float2 x = lane_xor(up ? h[k] : h[k + n], 4 * n), y = lane_xor(up ? l[k] : l[k + n], 4 * n);
+            const float2 z = n == 2 ? make_float2(0.0f, 0.0f) : lane_xor(up ? m[0] : m[1], 4);
+            h[k] = up ? h[k + n] : h[k];
+            l[k] = up ? l[k + n] : l[k];
+            if (n == 1) m[0] = up ? m[1] : m[0];
+            triple_add(h[k], l[k], m[k], x, y, z);
+        }
+    }
+    const bool up = (lane & 2) != 0;
+    const float x = lane_xor(up ? h[0].x : h[0].y, 2), y = lane_xor(up ? l[0].x : l[0].y, 2),
+                z = lane_xor(up ? m[0].x : m[0].y, 2);
+    float a = up ? h[0].y : h[0].x, b = up ? l[0].y : l[0].x, c = up ? m[0].y : m[0].x;
+    triple_add(a, b, c, x, y, z);
+    const float x1 = lane_xor(a, 1), y1 = lane_xor(b, 1), z1 = lane_xor(c, 1);
+    triple_add(a, b, c, x1, y1, z1);
+    const int slot = (lane >> 1) & 15;
+    if ((lane & 1) && slot < 12) w[slot] += double(a) + (double(b) + double(c));
 }
 
 // c2r pre-processing: Z[k] = (X[k] + X*[m]) + i (X[k] - X*[m]) w^{-k} with the

@@ -23,3 +23,8 @@ def program_output(source, tmp_path, *args):
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, (r.returncode, r.stdout, r.stderr)
     return r.stdout
+
+
+def shared_library(source, folder, *args):
+    """A shared library of kernels and their C entry points, for ctypes."""
+    return _compile(source, folder / "kernels.so", ("-shared", "-cudart", "static", *args))
