@@ -19,6 +19,7 @@
 
 #include "../../include/flusi.h"
 #include "kernels.cuh"
+#include "tuning.cuh"
 
 using namespace flusi;
 
@@ -80,6 +81,14 @@ thread_local std::string g_create_err;
 }  // namespace
 
 void flusi::set_global_error(const char* msg) { g_create_err = msg; }
+
+const flusi::TuneKnob flusi::tune_knobs[flusi::kTuneKnobs] = {
+    {&flusi_tuning::y_plan, {"yinv", "yfwd"}},
+    {&flusi_tuning::y_pair, {"yinv", "yfwd"}},
+    {&flusi_tuning::y_cols, {"yinv", "yfwd"}},
+    {&flusi_tuning::zf_plan, {"zinv_curl", "zfwd"}},   // FP32: it decides which kernel runs in both
+    {&flusi_tuning::z_cols, {"zinv_curl", "zfwd"}},
+    {&flusi_tuning::x_kernel, {"xpass_phys", "sponge_x"}}};
 
 namespace {
 
@@ -1303,17 +1312,7 @@ int flusi_autotune(flusi_t h, int steps, const char* cache_path, flusi_tuning* o
     rc = flusi_save(h, saved.get(), bytes);
     if (rc) return rc;
     flusi_get_tuning(h, &best);
-    struct Knob {
-        int flusi_tuning::*field;
-        const char* kernels[2];
-    };
-    const Knob knobs[] = {{&flusi_tuning::y_plan, {"yinv", "yfwd"}},
-                          {&flusi_tuning::y_pair, {"yinv", "yfwd"}},
-                          {&flusi_tuning::y_cols, {"yinv", "yfwd"}},
-                          {&flusi_tuning::zf_plan, {"zfwd", nullptr}},
-                          {&flusi_tuning::z_cols, {"zinv_curl", "zfwd"}},
-                          {&flusi_tuning::x_kernel, {"xpass_phys", "sponge_x"}}};
-    for (const Knob& kb : knobs) {
+    for (const TuneKnob& kb : tune_knobs) {
         // candidate values: the plans, or the default tile and two halvings
         std::vector<int> vals;
         if (kb.field == &flusi_tuning::y_plan || kb.field == &flusi_tuning::zf_plan) vals = {1, 0, 2};

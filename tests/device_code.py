@@ -12,7 +12,7 @@ def _compile(source, out, args):
     src = os.path.splitext(str(out))[0] + ".cu"
     with open(src, "w") as f:
         f.write(source)
-    r = subprocess.run([b.nvcc(), *b.ARCH, *b.FLAGS, "-I", CSRC, *args, src, "-o", str(out)], capture_output=True, text=True)
+    r = subprocess.run([b.nvcc(), *b.ARCH, *b.FLAGS, "-I", CSRC, src, "-o", str(out), *args], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return str(out)
 
