@@ -546,6 +546,20 @@ size_t real_size(int where, int prec)
 
 }  // namespace
 
+std::string flusi::tuning_signature(flusi_t h)
+{
+    flusi_tuning got{};
+    flusi_get_tuning(h, &got);
+    const int fp64 = h->prec == FLUSI_FP64;
+    std::string sig;
+    for (int i = 0; i < FLUSI_MAX_STAGES; ++i)
+        sig += std::to_string(got.y_radix[i]) + "," + std::to_string(got.zf_radix[i]) + ",";
+    for (int v : {got.y_tile_cols, got.z_tile_cols, ypass_kernel(fp64, h->g), zinv_kernel(fp64, h->g), zfwd_kernel(fp64, h->g),
+                  xpass_kernel(fp64, h->g)})
+        sig += std::to_string(v) + ",";
+    return sig;
+}
+
 extern "C" {
 
 void flusi_default_options(flusi_options* o)
@@ -1338,14 +1352,7 @@ int flusi_autotune(flusi_t h, int steps, const char* cache_path, flusi_tuning* o
             t.*kb.field = v;
             rc = flusi_set_tuning(h, &t);
             if (rc) break;
-            // settings that give the same plans, tiles and kernels are timed once
-            flusi_tuning got{};
-            flusi_get_tuning(h, &got);
-            std::string sig;
-            for (int i = 0; i < FLUSI_MAX_STAGES; ++i)
-                sig += std::to_string(got.y_radix[i]) + "," + std::to_string(got.zf_radix[i]) + ",";
-            sig += std::to_string(got.y_tile_cols) + "," + std::to_string(got.z_tile_cols) + "," +
-                   std::to_string(xpass_kernel(h->prec == FLUSI_FP64, h->g)) + "," + std::to_string(got.y_paired);
+            const std::string sig = tuning_signature(h);
             if (std::find(seen.begin(), seen.end(), sig) != seen.end()) continue;
             seen.push_back(sig);
             double ms = 0;

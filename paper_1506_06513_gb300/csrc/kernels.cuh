@@ -79,6 +79,11 @@ cudaError_t launch_zcol_inv(int cols, const float2* U, float2* W, const Geom& g,
 cudaError_t configure_zcol();
 // 1 when the y passes of this grid take the paired kernel (Geom::ypair)
 int ypass_paired(int fp64, const Geom& g);
+// which kernels run the y passes, the inverse and the forward z pass: 0 the staged,
+// 1 the paired (y) or the one by fields (inverse z), 2 the two-pass
+int ypass_kernel(int fp64, const Geom& g);
+int zinv_kernel(int fp64, const Geom& g);
+int zfwd_kernel(int fp64, const Geom& g);
 
 // z transforms (zpass.cu)
 //   zinv: U -> W[0..nf) in A form; nf = 3 (u) or 6 (u and omega = i k x u).

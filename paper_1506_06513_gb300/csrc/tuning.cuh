@@ -1,6 +1,8 @@
 // The autotuner's settings (flusi_autotune in flusi_capi.cu).
 #pragma once
 
+#include <string>
+
 #include "../../include/flusi.h"
 
 namespace flusi {
@@ -13,5 +15,9 @@ struct TuneKnob {
 };
 constexpr int kTuneKnobs = 6;
 extern const TuneKnob tune_knobs[kTuneKnobs];   // in the order of the descent
+
+// What a handle's settings run: plans, tiles and the kernel of every pass.  Settings
+// of one signature launch the same kernels and are timed once.
+std::string tuning_signature(flusi_t h);
 
 }  // namespace flusi

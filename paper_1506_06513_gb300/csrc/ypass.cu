@@ -449,6 +449,10 @@ cudaError_t launch_ypass(int fp64, bool inverse, void* W, const Geom& g, const F
 }
 
 int ypass_paired(int fp64, const Geom& g) { return fp64 ? y_paired<double>(g) : y_paired<float>(g); }
+int ypass_kernel(int fp64, const Geom& g)
+{
+    return ypass_paired(fp64, g) ? 1 : !fp64 && y_two_pass<float>(g) ? 2 : 0;
+}
 
 cudaError_t configure_ypass()
 {

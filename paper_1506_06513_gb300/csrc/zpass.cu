@@ -878,6 +878,11 @@ cudaError_t launch_zu(int mode, const void* Nh, void* U, void* H, const Geom& g,
 }  // namespace
 
 int zpass_tile_cols(int fp64, const Geom& g) { return fp64 ? zinv_tx<double>(g) : zinv_tx<float>(g); }
+int zfwd_kernel(int fp64, const Geom& g) { return !fp64 && z_two_pass<float>(g) ? 2 : 0; }
+int zinv_kernel(int fp64, const Geom& g)
+{
+    return (fp64 ? z_by_field<double>(g) : z_by_field<float>(g)) ? 1 : zfwd_kernel(fp64, g);
+}
 
 cudaError_t prepare_zmaps(int fp64, void* U, void* Ut, void* W, const Geom& g, ZMaps* maps)
 {

@@ -40,3 +40,54 @@ int main()
         timed.setdefault(name, set()).add(kernel)
     assert timed["y_plan"] == {"yinv", "yfwd"}
     assert timed["zf_plan"] == {"zinv_curl", "zfwd"}
+
+
+SIGNATURES = HEAD + r"""
+int main()
+{
+    const double L[3] = {1.0, 1.0, 1.0};
+    const int n[][3] = {%s};
+    for (auto& m : n) {
+        flusi_t h = nullptr;
+        if (flusi_create(m[0], m[1], m[2], L, 0.01, 1e-2, %s, &h) != FLUSI_OK) return 1;
+        for (int y = 0; y < 3; ++y)
+            for (int z = 0; z < 3; ++z)
+                for (int x = 0; x < 2; ++x) {
+                    flusi_tuning t{};
+                    t.y_plan = y, t.zf_plan = z, t.x_kernel = x;
+                    if (flusi_set_tuning(h, &t) != FLUSI_OK) return 2;
+                    printf("%%d %%d %%d %%d %%d %%d %%s\n", m[0], m[1], m[2], y, z, x, tuning_signature(h).c_str());
+                }
+        flusi_destroy(h);
+    }
+    return 0;
+}
+"""
+
+
+def _signatures(library, tmp_path, grids, prec):
+    text = SIGNATURES % (", ".join("{%d, %d, %d}" % g for g in grids), prec)
+    out = {}
+    for line in program_output(text, tmp_path, *library).splitlines():
+        *k, sig = line.split()
+        k = tuple(map(int, k))
+        out[k[:3], k[3:]] = sig
+    return out
+
+
+def test_two_pass_and_staged_kernels_are_told_apart(library, tmp_path):
+    """At 64, 192, 384 and 512 rows plans 0 and 1 have the same radices; in FP32
+    plan 1 runs the two-pass kernels and plan 0 the staged ones."""
+    grids = [(96, n, n) for n in (64, 192, 384, 512)]
+    sig = _signatures(library, tmp_path, grids, "FLUSI_FP32")
+    for g in grids:
+        assert sig[g, (0, 1, 0)] != sig[g, (1, 1, 0)] and sig[g, (1, 0, 0)] != sig[g, (1, 1, 0)], g
+        assert sig[g, (1, 1, 0)] != sig[g, (1, 1, 1)], g
+        # the staged kernels with the same radices stay one setting
+        if sig[g, (0, 0, 0)].split(",")[:2] == sig[g, (2, 2, 0)].split(",")[:2] and g[1] in (64, 512):
+            assert sig[g, (0, 0, 0)] == sig[g, (2, 2, 0)], g
+    # without two-pass kernels (FP64; 48 and 729 rows), equal radices are one setting
+    sig = _signatures(library, tmp_path, [(96, 512, 64)], "FLUSI_FP64")
+    assert sig[(96, 512, 64), (0, 0, 0)] == sig[(96, 512, 64), (1, 1, 0)] == sig[(96, 512, 64), (2, 2, 0)]
+    sig = _signatures(library, tmp_path, [(96, 48, 729)], "FLUSI_FP32")
+    assert sig[(96, 48, 729), (1, 0, 0)] == sig[(96, 48, 729), (1, 1, 0)]
