@@ -376,7 +376,8 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * undrained force rows are dropped, as by flusi_load.  cache_path (NULL: no
  * cache) names a text file of lines "key y_plan zf_plan y_cols z_cols
  * x_kernel y_pair", key = GPU name (spaces as '_'), SM count, grid, precision,
- * time scheme and wake terms: a line with this handle's key is applied
+ * time scheme, wake terms, 2/3 rule and flusi_build_id (what is best depends
+ * on the kernels): a line with this handle's key is applied
  * without timing; otherwise the result is appended (a file that cannot be
  * written is FLUSI_EINVAL after the tuning is applied).  *out (may be
  * NULL) receives the chosen settings as flusi_get_tuning does.  The saved

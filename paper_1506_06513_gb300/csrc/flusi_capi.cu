@@ -546,6 +546,25 @@ size_t real_size(int where, int prec)
 
 }  // namespace
 
+std::string flusi::tuning_key(flusi_t h)
+{
+    int dev = 0;
+    cudaDeviceProp prop{};
+    cudaGetDevice(&dev);
+    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) cudaGetLastError();
+    std::string name = prop.name;
+    for (char& c : name)
+        if (c == ' ' || c == '\t') c = '_';
+    const bool wake = h->opt.sponge_c > 0 || h->opt.layer_width[0] > 0 || h->opt.layer_width[1] > 0 ||
+                      h->opt.layer_width[2] > 0;
+    char buf[256];
+    std::snprintf(buf, sizeof buf, "%s|%d|%dx%dx%d|%s|%s|%s|d%d|%s", name.empty() ? "gpu" : name.c_str(),
+                  prop.multiProcessorCount, h->nx, h->ny, h->nz,
+                  h->prec == FLUSI_FP64 ? "fp64" : h->prec == FLUSI_FP32 ? "fp32" : h->prec == FLUSI_FP32_SPLITBF16 ? "bf16x2" : "bf16x3",
+                  is_rk4(h) ? "rk4" : "ab2", wake ? "wake" : "nowake", h->opt.dealias_strict, flusi_build_id());
+    return buf;
+}
+
 std::string flusi::tuning_signature(flusi_t h)
 {
     flusi_tuning got{};
@@ -1215,25 +1234,6 @@ int time_kernels(flusi_t h, int steps, const char* const names[2], double* ms_ou
     }
     *ms_out = sum;
     return FLUSI_OK;
-}
-
-std::string tuning_key(flusi_t h)
-{
-    int dev = 0;
-    cudaDeviceProp prop{};
-    cudaGetDevice(&dev);
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) cudaGetLastError();
-    std::string name = prop.name;
-    for (char& c : name)
-        if (c == ' ' || c == '\t') c = '_';
-    const bool wake = h->opt.sponge_c > 0 || h->opt.layer_width[0] > 0 || h->opt.layer_width[1] > 0 ||
-                      h->opt.layer_width[2] > 0;
-    char buf[256];
-    std::snprintf(buf, sizeof buf, "%s|%d|%dx%dx%d|%s|%s|%s|d%d", name.empty() ? "gpu" : name.c_str(),
-                  prop.multiProcessorCount, h->nx, h->ny, h->nz,
-                  h->prec == FLUSI_FP64 ? "fp64" : h->prec == FLUSI_FP32 ? "fp32" : h->prec == FLUSI_FP32_SPLITBF16 ? "bf16x2" : "bf16x3",
-                  is_rk4(h) ? "rk4" : "ab2", wake ? "wake" : "nowake", h->opt.dealias_strict);
-    return buf;
 }
 
 // the last line of the cache with this key, if any

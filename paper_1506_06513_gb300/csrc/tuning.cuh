@@ -19,5 +19,7 @@ extern const TuneKnob tune_knobs[kTuneKnobs];   // in the order of the descent
 // What a handle's settings run: plans, tiles and the kernel of every pass.  Settings
 // of one signature launch the same kernels and are timed once.
 std::string tuning_signature(flusi_t h);
+// The key of a handle's line in a tuning cache.
+std::string tuning_key(flusi_t h);
 
 }  // namespace flusi

@@ -91,3 +91,24 @@ def test_two_pass_and_staged_kernels_are_told_apart(library, tmp_path):
     assert sig[(96, 512, 64), (0, 0, 0)] == sig[(96, 512, 64), (1, 1, 0)] == sig[(96, 512, 64), (2, 2, 0)]
     sig = _signatures(library, tmp_path, [(96, 48, 729)], "FLUSI_FP32")
     assert sig[(96, 48, 729), (1, 0, 0)] == sig[(96, 48, 729), (1, 1, 0)]
+
+
+def test_cache_lines_belong_to_one_build(library, tmp_path):
+    """Which setting is best depends on the kernels, so a line of another build
+    does not apply: the key ends in the library's source hash."""
+    out = program_output(HEAD + r"""
+int main()
+{
+    const double L[3] = {1.0, 1.0, 1.0};
+    flusi_t h = nullptr;
+    if (flusi_create(96, 64, 512, L, 0.01, 1e-2, FLUSI_FP32, &h) != FLUSI_OK) return 1;
+    printf("%s\n", tuning_key(h).c_str());
+    return flusi_destroy(h);
+}
+""", tmp_path, *library)
+    from conftest import build_flusi
+    build_flusi()
+    from paper_1506_06513_gb300 import _build
+    key = out.strip()
+    assert "96x64x512|fp32|ab2|nowake" in key and " " not in key
+    assert key.split("|")[-1] == _build.source_hash()
