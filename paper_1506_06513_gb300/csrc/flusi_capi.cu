@@ -314,6 +314,13 @@ int* status_word(flusi_t h) { return &reinterpret_cast<StepState*>(h->ws + h->os
 // x round trip of the vorticity.
 bool sponge_kernel(flusi_t h) { return has_sponge(h) && !xpass_fuses_sponge(h->prec == FLUSI_FP64, h->g); }
 
+// Rows of partial sums of the physical x pass.  The sponge decides between kernels,
+// so it is counted again when the options change.
+int step_xgrid(flusi_t h)
+{
+    return std::min(xpass_grid(h->prec == FLUSI_FP64, h->g, has_sponge(h) && !sponge_kernel(h)), h->part_cap);
+}
+
 // Kernels per step: per right-hand side kinematics, z inverse, y inverse, x
 // pass, (sponge x pass), y forward, z forward, update; the scalar kernel once.
 int step_kernels(flusi_t h) { return (is_rk4(h) ? 4 : 1) * (7 + (sponge_kernel(h) ? 1 : 0)) + 1; }
@@ -643,6 +650,7 @@ int flusi_set_options(flusi_t h, const flusi_options* o)
     layout(h);
     drop_graph(h);
     if (h->bound) {
+        h->xgrid = step_xgrid(h);
         int rc = prepare_maps(h);
         if (rc) return rc;
     }
@@ -680,10 +688,9 @@ int flusi_bind(flusi_t h, void* ws, size_t bytes, void* stream)
     h->ws = static_cast<char*>(ws);
     h->ws_bytes = bytes;
     h->stream = static_cast<cudaStream_t>(stream);
-    h->xgrid = xpass_grid(h->prec == FLUSI_FP64, h->g);
+    h->xgrid = step_xgrid(h);
     int rc = prepare_maps(h);
     if (rc) return rc;
-    if (h->xgrid > h->part_cap) h->xgrid = h->part_cap;
     CK(cudaMemsetAsync(h->ws, 0, h->total, h->stream), "clear workspace");
     auto tx = twiddles(h->nx), ty = twiddles(h->ny), tz = twiddles(h->nz);
     auto fx = twiddles32(tx), fy = twiddles32(ty), fz = twiddles32(tz);
@@ -1302,7 +1309,7 @@ int flusi_set_tuning(flusi_t h, const flusi_tuning* t)
     CK(cudaMemcpyAsync(h->ws + h->opz, pz.data(), sizeof(int) * pz.size(), cudaMemcpyHostToDevice, h->stream),
        "digit reversal");
     CK(cudaStreamSynchronize(h->stream), "retune tables");
-    h->xgrid = std::min(xpass_grid(h->prec == FLUSI_FP64, h->g), h->part_cap);
+    h->xgrid = step_xgrid(h);
     return prepare_maps(h);
 }
 

@@ -1076,10 +1076,10 @@ template <typename T, int R, int S> size_t sq_smem(const Geom& g, bool sponge = 
 // points (phys_line).
 template <typename T, int R> constexpr bool sq_plain() { return sizeof(T) == 8 || R != 8; }
 
-// grid = the virtual CTAs (rows of partial sums, x_grid, whichever kernel it was
-// counted for); a batch of n members runs about one resident wave in all, each CTA taking several
-// virtual ones, instead of n full grids of CTAs that each take one or two
-// tiles and pay their table and frame loads for them.
+// grid = the virtual CTAs (rows of partial sums, x_grid); a batch of n members runs
+// about one resident wave in all, each CTA taking several virtual ones, instead of n
+// full grids of CTAs that each take one or two tiles and pay their table and frame
+// loads for them.
 template <typename T, int R, int S>
 void launch_sq(bool layer, bool sponge, cplx<T>* w, const Geom& g, const double2* tw, const XExtra& ex0,
                const StepState* st, cudaStream_t s, int grid)
@@ -1158,16 +1158,21 @@ template <typename T> size_t x_smem(const Geom& g, int lgRB, int NF)
     return s;
 }
 
-template <typename T> int x_grid(const Geom& g)
+// CTAs of the physical pass, from the occupancy of the kernel that runs it; with the
+// fused sponge of the same kernel without it where that exists, else (256, 128 and 64
+// points in FP32) of the fused one: counted for the line kernel that takes those
+// lengths without the sponge, the pass took 89.9 us in place of 88.0 at 256 x 128 x
+// 128, 51.3 and 49.2 at 128^3, 67.5 and 65.6 at 64 x 256 x 256, 321 and 322 at 256^3.
+template <typename T> int x_grid(const Geom& g, bool sponge)
 {
     const int sm_count = sm_count_here();
     int per_sm = 0, ntiles = 0;
     const int kind = sq_kind<T>(g);
-    const XLineOps* line = phys_line<T>(g, false);
+    const XLineOps* line = phys_line<T>(g, sponge);
 #define FLUSI_SQ_OCC(R, S)                                                                          \
     ntiles = ceil_div(g.nz * g.ny, sq_rows<sq_lanes<R, S>()>());                                               \
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, !sq_plain<T, R>()>, 192, \
-                                                  sq_smem<T, R, S>(g));
+                                                  sq_smem<T, R, S>(g, !sq_plain<T, R>()));
     if (line) {
         ntiles = ceil_div(g.nz * g.ny, line->rows);
         per_sm = line->phys_per_sm();
@@ -1218,7 +1223,7 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
         if (mode == XP_PHYS && phys_line<T>(g, sponge)) {
             const Batch& B = current_batch();
             XExtra e = ex;
-            e.nvirt = x_grid<T>(g);
+            e.nvirt = x_grid<T>(g, sponge);
             // a batch of n members runs about one resident wave in all (launch_sq)
             const int resident = sm_count_here() * std::max(1, line->phys_per_sm());
             const int run = B.n > 1 ? std::min(e.nvirt, std::max(1, ceil_div(resident, B.n))) : e.nvirt;
@@ -1229,14 +1234,14 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
     switch (mode) {
     case XP_PHYS:
         switch (sq_kind<T>(g)) {
-        case 161: launch_sq<T, 16, 1>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
-        case 81: launch_sq<T, 8, 1>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
-        case 162: launch_sq<T, 16, 2>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
-        case 82: launch_sq<T, 8, 2>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
-        case 120: launch_sq<T, 12, 0>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
-        case 80: launch_sq<T, 8, 0>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g)); break;
+        case 161: launch_sq<T, 16, 1>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
+        case 81: launch_sq<T, 8, 1>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
+        case 162: launch_sq<T, 16, 2>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
+        case 82: launch_sq<T, 8, 2>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
+        case 120: launch_sq<T, 12, 0>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
+        case 80: launch_sq<T, 8, 0>(layer, sponge, w, g, tw, ex, st, s, x_grid<T>(g, sponge)); break;
         default:
-            k_xpass<T, XP_PHYS><<<dim3(x_grid<T>(g), 1, current_batch().n), kThreadsX, smem, s>>>(
+            k_xpass<T, XP_PHYS><<<dim3(x_grid<T>(g, sponge), 1, current_batch().n), kThreadsX, smem, s>>>(
                 w, g, plan, tw, pos, ex, lg, st, current_batch().mb);
         }
         break;
@@ -1258,10 +1263,10 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
 
 }  // namespace
 
-int xpass_grid(int fp64, const Geom& g)
+int xpass_grid(int fp64, const Geom& g, int sponge_fused)
 {
     if (!fp64 && g.xtc) return xpass_tc_grid(g);
-    return fp64 ? x_grid<double>(g) : x_grid<float>(g);
+    return fp64 ? x_grid<double>(g, sponge_fused) : x_grid<float>(g, sponge_fused);
 }
 
 // 1 when the physical x pass (square kernel) forms and transforms chi_sp omega itself
