@@ -338,18 +338,21 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  * 8 8 4 (256 = 16 16).  The inverse z pass always takes plan 0 (its kernel
  * has no radix-16 variant).  In FP32, plan 1 with the widest tiles takes the
  * two-pass kernels (n = R L in two register passes) at the lengths that have
- * them (most of 64..1024) in place of the radices reported.
+ * them (every length from 64 to 1024 but 729 and 972; z over 512 rows on grids
+ * of enough columns) in place of the radices reported.
  * Tile columns (y_cols, z_cols): 0 (default) the widest tile that fits a
  * block's 64 KB (two-pass kernels over 512 rows: 16 columns, 128 KB; on grids
- * whose widest tiles would not fill the GPU, a narrower one), else a cap on the tile's columns (x columns times z planes
- * for y; columns of the flattened (y, x) plane for z), a power of two of at
- * least 32 bytes of complex values (4 in FP32, 2 in FP64) and at most 256.
+ * whose widest tiles would not fill the GPU, a narrower one), else a cap on the
+ * tile's columns (x columns times z planes for y; columns of the flattened (y, x)
+ * plane for z), a power of two of at least 32 bytes of complex values (4 in FP32,
+ * 2 in FP64) and at most 256.
  * Grids under 2^14 values of kept columns (My Mxp nz; FP64 2^15) take their
- * inverse z pass a block per column range and field, whatever the plan.
- * x_kernel: 0 (default) the register-resident line kernel where one exists
- * (nx = 128, 256, 512, 1024, and its rectangular form at nx = 64, 96; in FP32
- * the general line kernels at every other length from 16 on), 1 the
- * shared-memory kernel of every length.
+ * inverse z pass a block per column range and field, whatever zf_plan says.
+ * x_kernel: 0 (default) a register-resident line kernel where one exists:
+ * those of their own at nx = 128, 256, 512, 1024 and (rectangular) 64, 96; in
+ * FP32 the general line kernels at every other length from 16 on, and at 256,
+ * 128 and 64 unless the step has the vorticity sponge.  1 the shared-memory
+ * kernel of every length.
  * y_pair: 1 the y passes' paired kernel, a cluster of two CTAs per tile,
  * each holding the grid rows of one parity and transforming them at half the
  * length, joined by a radix-2 step through distributed shared memory, so
@@ -358,8 +361,9 @@ int flusi_kernels_per_step(flusi_t h, int *count);
  *
  * flusi_get_tuning fills every field, including the read-only ones: the
  * radices each pass takes (0-terminated), the columns a tile takes, and
- * whether the x pass runs the register-resident kernel that also forms the
- * sponge term (1 at the six lengths named first, 0 for the general kernels).
+ * whether the x pass forms the sponge term itself where a step has one
+ * (x_line_kernel: 1 at the six lengths that have a line kernel of their own, 0
+ * elsewhere and for x_kernel 1).
  * flusi_set_tuning takes the six settings (the rest is ignored); any
  * other value is FLUSI_EINVAL with nothing changed.  On a bound handle it
  * waits for the handle's stream, uploads the new digit-reversal tables and

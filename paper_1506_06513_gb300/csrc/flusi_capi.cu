@@ -581,7 +581,7 @@ std::string flusi::tuning_signature(flusi_t h)
     for (int i = 0; i < FLUSI_MAX_STAGES; ++i)
         sig += std::to_string(got.y_radix[i]) + "," + std::to_string(got.zf_radix[i]) + ",";
     for (int v : {got.y_tile_cols, got.z_tile_cols, ypass_kernel(fp64, h->g), zinv_kernel(fp64, h->g), zfwd_kernel(fp64, h->g),
-                  xpass_kernel(fp64, h->g)})
+                  xpass_kernel(fp64, h->g, has_sponge(h) && !sponge_kernel(h))})
         sig += std::to_string(v) + ",";
     return sig;
 }

@@ -152,9 +152,9 @@ struct XExtra {
     int nvirt;
 };
 int xpass_fuses_sponge(int fp64, const Geom& g);
-// 0 the shared-memory kernel, 1 a line kernel of xpass.cu, 2 the general line
-// kernels of xline.cuh (FP32)
-int xpass_kernel(int fp64, const Geom& g);
+// which kernel runs the physical pass: 0 the shared-memory kernel, 1 a line kernel of
+// xpass.cu, 2 the general line kernels of xline.cuh (FP32)
+int xpass_kernel(int fp64, const Geom& g, int sponge_fused);
 int xpass_grid(int fp64, const Geom& g, int sponge_fused);   // CTAs of the persistent physical pass
 cudaError_t launch_xpass(int fp64, int mode, void* W, const Geom& g, const FftPlan& plan,
                          const double2* tw, const int* pos, const XExtra& ex, const StepState* st,

@@ -1276,10 +1276,10 @@ int xpass_fuses_sponge(int fp64, const Geom& g)
     return fp64 ? sq_kind<double>(g) != 0 : sq_kind<float>(g) != 0;
 }
 
-int xpass_kernel(int fp64, const Geom& g)
+int xpass_kernel(int fp64, const Geom& g, int sponge_fused)
 {
-    if (fp64 ? sq_kind<double>(g) != 0 : sq_kind<float>(g) != 0) return 1;
-    return !fp64 && xline_of<float>(g) ? 2 : 0;
+    if (!fp64 && phys_line<float>(g, sponge_fused)) return 2;
+    return fp64 ? sq_kind<double>(g) != 0 : sq_kind<float>(g) != 0;
 }
 
 cudaError_t launch_xpass(int fp64, int mode, void* W, const Geom& g, const FftPlan& plan,
