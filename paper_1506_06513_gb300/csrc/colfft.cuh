@@ -182,11 +182,12 @@ struct ColState {
 // landed and been read), then for the landing; both waits are bounded.  A group
 // that gives up reports FLUSI_ETIMEOUT and leaves its loop; what it no longer
 // sends lets the other one's wait run out too, and the block then waits (bounded)
-// for every load in flight before it ends.
+// for every TMA load in flight, and each thread for its own copies, before it ends.
+// limit: of a wait, in SM clocks (as mbar_wait).
 template <class X, class Job>
-__device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, int* err, Job& job)
+__device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, int* err, Job& job,
+                                         const long long limit = 400000000LL)
 {
-    constexpr long long kLimit = 400000000LL;   // SM clocks, as mbar_wait
     constexpr int CH = X::CH;
     const int group = X::GROUPS == 1 ? 0 : (threadIdx.x >= X::T ? 1 : 0), tid = threadIdx.x & (X::T - 1);
     auto slot_of = [](int s) { return X::BUFS == 1 ? 0 : s % X::BUFS; };
@@ -225,8 +226,8 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
         for (int h = 0; h < CH; ++h) {
             const int s = i * CH + h, load = s / X::BUFS;
             const long long t0 = clock64();
-            while (ok && *(volatile int*)&sh.issued[slot_of(s)] <= load) ok = clock64() - t0 <= kLimit;
-            if (ok) ok = mbar_wait(sh.full + slot_of(s), (unsigned)load & 1u, kLimit);
+            while (ok && *(volatile int*)&sh.issued[slot_of(s)] <= load) ok = clock64() - t0 <= limit;
+            if (ok) ok = mbar_wait(sh.full + slot_of(s), (unsigned)load & 1u, limit);
         }
         if (!ok) {
             *(volatile int*)&sh.bad[group] = 1;
@@ -257,10 +258,11 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
             }
         });
     }
+    if (!tma) cp_async_wait_all();
     __syncthreads();
     if (tma && threadIdx.x == 0 && (sh.bad[0] | sh.bad[1]))
         for (int b = 0; b < X::BUFS; ++b)
-            if (sh.issued[b] > 0) mbar_wait(sh.full + b, (unsigned)(sh.issued[b] - 1) & 1u, kLimit);
+            if (sh.issued[b] > 0) mbar_wait(sh.full + b, (unsigned)(sh.issued[b] - 1) & 1u, limit);
 }
 
 // The lengths served, X(n, R, L).  Others (and narrowed tiles, the other plans
