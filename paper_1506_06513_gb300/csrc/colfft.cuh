@@ -273,19 +273,12 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
     X(384, 24, 16) X(432, 27, 16) X(486, 27, 18) X(512, 32, 16) X(576, 24, 24) X(648, 24, 27)              \
     X(768, 32, 24) X(864, 32, 27) X(1024, 32, 32)
 
-inline int col_sms()
-{
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-}
 // Persistent grid of a kernel with `smem` bytes over `tiles` tiles per member.
 template <class X, class K> dim3 col_grid(K kernel, long long tiles)
 {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, X::THREADS, X::kSmem);
-    const long long n = current_batch().n, resident = (long long)col_sms() * (per_sm > 0 ? per_sm : 1);
+    const long long n = current_batch().n, resident = (long long)sm_count() * (per_sm > 0 ? per_sm : 1);
     const long long share = (resident + n - 1) / n;
     return dim3((unsigned)(tiles < share ? tiles : share), 1, (unsigned)n);
 }

@@ -58,9 +58,18 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C b)
     return r;
 }
 
-// SMs of the GB300: a pass whose widest tiles would leave some without a block
-// takes narrower ones.
+// SMs of the GB300, where a rule must not depend on the part (z_two_pass in zpass.cu:
+// which of two kernels that round differently).
 constexpr int kSMs = 152;
+// SMs of the current device: a pass whose widest tiles would leave some without a
+// block takes narrower ones, and persistent grids fill them once.
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();   // (a handle without a device: the sizes it reports)
+    return sms > 0 ? sms : kSMs;
+}
 
 // Largest FFT length along any axis (the x transform runs at nx/2).
 constexpr int kMaxN = 1024;

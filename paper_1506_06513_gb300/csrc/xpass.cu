@@ -54,14 +54,6 @@ template <typename T> const XLineOps* xline_of(const Geom& g)
         });
     return found;
 }
-int sm_count_here()
-{
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-}
-
 constexpr int kThreadsX = 192;
 constexpr int kWarpsX = kThreadsX / 32;
 // complex elements per tile: 48 KiB of shared memory
@@ -1090,11 +1082,9 @@ void launch_sq(bool layer, bool sponge, cplx<T>* w, const Geom& g, const double2
     ex.nvirt = grid;
     int run = grid;
     if (B.n > 1) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass_sq<T, R, S, false, !sq_plain<T, R>()>, 192, smem);
-        const int resident = std::max(1, sms * std::max(1, per_sm));
+        const int resident = sm_count() * std::max(1, per_sm);
         run = std::min(grid, std::max(1, ceil_div(resident, B.n)));
     }
     const dim3 gd(run, 1, B.n);
@@ -1145,7 +1135,9 @@ template <typename T> int x_lgrb(const Geom& g)
     const int nh = g.nx / 2;
     int RB = 32;
     while (RB > 1 && nh * 6 * RB > tile_elems<T>()) RB >>= 1;
-    while (RB > 1 && ceil_div(g.nz * g.ny, RB) < kSMs) RB >>= 1;   // small grids: a tile for every SM (32^3 FP64: 32 tiles 94 us, 256 tiles 37 us)
+    // small grids: a tile for every SM (32^3 FP64: 32 tiles 94 us, 256 tiles 37 us)
+    const int sms = sm_count();
+    while (RB > 1 && ceil_div(g.nz * g.ny, RB) < sms) RB >>= 1;
     return __builtin_ctz(RB);
 }
 
@@ -1165,7 +1157,6 @@ template <typename T> size_t x_smem(const Geom& g, int lgRB, int NF)
 // 128, 51.3 and 49.2 at 128^3, 67.5 and 65.6 at 64 x 256 x 256, 321 and 322 at 256^3.
 template <typename T> int x_grid(const Geom& g, bool sponge)
 {
-    const int sm_count = sm_count_here();
     int per_sm = 0, ntiles = 0;
     const int kind = sq_kind<T>(g);
     const XLineOps* line = phys_line<T>(g, sponge);
@@ -1196,7 +1187,7 @@ template <typename T> int x_grid(const Geom& g, bool sponge)
     }
 #undef FLUSI_SQ_OCC
     if (per_sm <= 0) per_sm = 1;
-    int grid = sm_count * per_sm;
+    int grid = sm_count() * per_sm;
     return grid < ntiles ? grid : ntiles;
 }
 
@@ -1217,7 +1208,7 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
     if constexpr (sizeof(T) == 4) {
         const XLineOps* line = xline_of<T>(g);
         if (line && (mode == XP_R2C || mode == XP_C2R || mode == XP_SPONGE)) {
-            line->lines(mode, s, w, g, tw, ex, sm_count_here());
+            line->lines(mode, s, w, g, tw, ex, sm_count());
             return cudaGetLastError();
         }
         if (mode == XP_PHYS && phys_line<T>(g, sponge)) {
@@ -1225,7 +1216,7 @@ cudaError_t launch_x(int mode, void* W, const Geom& g, const FftPlan& plan, cons
             XExtra e = ex;
             e.nvirt = x_grid<T>(g, sponge);
             // a batch of n members runs about one resident wave in all (launch_sq)
-            const int resident = sm_count_here() * std::max(1, line->phys_per_sm());
+            const int resident = sm_count() * std::max(1, line->phys_per_sm());
             const int run = B.n > 1 ? std::min(e.nvirt, std::max(1, ceil_div(resident, B.n))) : e.nvirt;
             line->phys(dim3(run, 1, B.n), s, w, g, tw, e, st, B.mb);
             return cudaGetLastError();

@@ -685,16 +685,12 @@ int xpass_tc_supported(int nx) { return nx == 512 || nx == 256; }
 
 int xpass_tc_grid(const Geom& g)
 {
-    int dev = 0, sm_count = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-    if (sm_count <= 0) sm_count = 1;
     int per_sm = 1;
     if (g.nx == 512) per_sm = g.xtc == 3 ? tc_per_sm<16, 3>() : tc_per_sm<16, 2>();
     else per_sm = g.xtc == 3 ? tc_per_sm<8, 3>() : tc_per_sm<8, 2>();
     const int RB = 128 / (g.nx / 32);
     const int ntiles = ceil_div(g.nz * g.ny, RB);
-    const int grid = per_sm * sm_count;
+    const int grid = per_sm * sm_count();
     return grid < ntiles ? grid : ntiles;
 }
 

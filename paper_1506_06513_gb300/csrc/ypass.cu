@@ -273,15 +273,16 @@ template <typename T> YTile y_tile(const Geom& g, int ncomp)
     // y 32^3 FP64 23 us against 14, step of 48^3 196 and 172, FP32 60 and 54; 96 x
     // 48 x 64 388 and 351, 61 and 55)
     const long long runs = (long long)current_batch().n * ceil_div(g.Mxp, TX) * 6;
+    const int sms = sm_count();
     if (y_two_pass<T>(g)) {
         // the two-pass kernel's full tile, or one plane
         NP = ycol_full(g.ny) / TX;
-        if (NP > g.nz || runs * ceil_div(g.nz, NP) < kSMs) NP = 1;
+        if (NP > g.nz || runs * ceil_div(g.nz, NP) < sms) NP = 1;
     } else {
         const int cap = tile_elems<T>();
         while (TX > 1 && (g.ny * TX > cap || TX > cmax)) TX >>= 1;
         while (2 * NP * TX * g.ny <= cap && 2 * NP * TX <= std::min(kThreads, cmax) && 2 * NP <= g.nz) NP *= 2;
-        while (NP > 1 && runs * ceil_div(g.nz, NP) < kSMs) NP >>= 1;
+        while (NP > 1 && runs * ceil_div(g.nz, NP) < sms) NP >>= 1;
     }
     t.lgTX = __builtin_ctz(TX);
     t.lgNP = __builtin_ctz(NP);

@@ -704,14 +704,15 @@ template <typename T> int z_tx(const Geom& g, int fields)
     const int cmax = g.zcols > 0 ? g.zcols : 64;   // columns per tile
     const int Q = g.My * g.Mxp;
     const long long tiles = (long long)current_batch().n * fields;
+    const int sms = sm_count();
     if (z_two_pass<T>(g)) {
         const int full = zcol_full(g.nz);
-        return g.nz > 512 || tiles * ceil_div(Q, full) >= kSMs ? full : 8;
+        return g.nz > 512 || tiles * ceil_div(Q, full) >= sms ? full : 8;
     }
     int TX = sizeof(T) == 4 ? 16 : 8;
     while (TX > 1 && (g.nz * TX > cap_zi<T>() || TX > cmax)) TX >>= 1;
     while (2 * TX * g.nz <= cap_zi<T>() && 2 * TX <= cmax) TX *= 2;
-    while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(Q, TX) < kSMs) TX >>= 1;
+    while (TX > (sizeof(T) == 4 ? 4 : 2) && tiles * ceil_div(Q, TX) < sms) TX >>= 1;
     return TX;
 }
 template <typename T> int zinv_tx(const Geom& g) { return z_tx<T>(g, 1); }
@@ -734,8 +735,9 @@ template <typename T> bool z_by_field(const Geom& g)
 template <typename T> int zfield_tx(const Geom& g, int nf)
 {
     int TX = sizeof(T) == 4 ? 16 : 8;
+    const int sms = sm_count();
     while (TX > 2 && (g.nz * TX > cap_zi<T>() || (g.zcols > 0 && TX > g.zcols) ||
-                      (long long)current_batch().n * nf * ceil_div(g.My * g.Mxp, TX) < kSMs))
+                      (long long)current_batch().n * nf * ceil_div(g.My * g.Mxp, TX) < sms))
         TX >>= 1;
     return TX;
 }
