@@ -70,13 +70,13 @@ cudaError_t launch_ypass(int fp64, bool inverse, void* W, const Geom& g, const F
 int ycol_full(int ny);
 cudaError_t launch_ycol(bool inverse, int cols, float2* W, const Geom& g, const double2* tw, int ncomp, const StepState* st,
                         const CUtensorMap& map, int bh, int* err, cudaStream_t s);
-cudaError_t configure_ycol();
+cudaError_t configure_ycol(int ny);
 int zcol_full(int nz);
 cudaError_t launch_zcol_fwd(int cols, float2* W, int nf, const Geom& g, const double2* tw, const StepState* st,
                             const CUtensorMap& map, int bh, int* err, cudaStream_t s);
 cudaError_t launch_zcol_inv(int cols, const float2* U, float2* W, const Geom& g, const double2* tw, int nf,
                             const StepState* st, const CUtensorMap& map, int bh, int* err, cudaStream_t s);
-cudaError_t configure_zcol();
+cudaError_t configure_zcol(int nz);
 // 1 when the y passes of this grid take the paired kernel (Geom::ypair)
 int ypass_paired(int fp64, const Geom& g);
 // which kernels run the y passes, the inverse and the forward z pass: 0 the staged,
@@ -172,9 +172,11 @@ cudaError_t configure_xpass_tc();
 // Message returned by flusi_last_error(NULL).
 void set_global_error(const char* msg);
 
-// Shared-memory limits of every instantiation (once per process and device).
+// Shared-memory limits of every instantiation (once per process and device), and of
+// the FP32 kernels made for a length (once more per length; configure_ycol, _zcol).
 cudaError_t configure_ypass();
 cudaError_t configure_zpass();
 cudaError_t configure_xpass();
+cudaError_t configure_xline(int nx);
 
 }  // namespace flusi

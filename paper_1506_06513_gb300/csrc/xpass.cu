@@ -1285,14 +1285,19 @@ cudaError_t launch_xpass(int fp64, int mode, void* W, const Geom& g, const FftPl
                 : launch_x<float>(mode, W, g, plan, tw, pos, ex, st, s);
 }
 
+cudaError_t configure_xline(int nx)
+{
+    cudaError_t e = cudaSuccess;
+    each_xline([&](const XLineOps& o) {
+        if (!e && o.nx == nx) e = o.configure();
+    });
+    return e;
+}
+
 cudaError_t configure_xpass()
 {
     const int big = 200 * 1024;
-    cudaError_t e = cudaSuccess;
-    each_xline([&](const XLineOps& o) {
-        if (!e) e = o.configure();
-    });
-    if (e) return e;
+    cudaError_t e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
     FLUSI_SMEM((k_xpass<float, XP_PHYS>))

@@ -171,7 +171,7 @@ cudaError_t launch_ycol(bool inverse, int cols, float2* W, const Geom& g, const 
     }
 }
 
-cudaError_t configure_ycol()
+cudaError_t configure_ycol(int ny)
 {
     cudaError_t e = cudaSuccess;
     auto one = [&](const void* kernel, size_t smem) {
@@ -180,15 +180,18 @@ cudaError_t configure_ycol()
 #define FLUSI_KERNELS(X)                                       \
     one((const void*)k_ycol<X, true>, X::kSmem);               \
     one((const void*)k_ycol<X, false>, X::kSmem);
+    switch (ny) {
 #define FLUSI_CASE(n, R, L)                                    \
-    {                                                          \
+    case n: {                                                  \
         using Full = Col<R, L, y_cols<n>()>;                   \
         using Small = Col<R, L, kTX>;                          \
         FLUSI_KERNELS(Full)                                    \
         FLUSI_KERNELS(Small)                                   \
+        break;                                                 \
     }
-    FLUSI_COL_LENGTHS(FLUSI_CASE)
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
+    }
 #undef FLUSI_KERNELS
     return e;
 }

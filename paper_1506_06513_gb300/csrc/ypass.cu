@@ -458,8 +458,7 @@ int ypass_kernel(int fp64, const Geom& g)
 cudaError_t configure_ypass()
 {
     const int big = 100 * 1024;
-    cudaError_t e = configure_ycol();
-    if (e) return e;
+    cudaError_t e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
 #define FLUSI_SMEM_Y(T, R16)                         \

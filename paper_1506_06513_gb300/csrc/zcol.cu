@@ -364,7 +364,7 @@ cudaError_t launch_zcol_inv(int cols, const float2* U, float2* W, const Geom& g,
     }
 }
 
-cudaError_t configure_zcol()
+cudaError_t configure_zcol(int nz)
 {
     cudaError_t e = cudaSuccess;
     auto one = [&](const void* kernel, size_t smem) {
@@ -373,15 +373,18 @@ cudaError_t configure_zcol()
 #define FLUSI_KERNELS(X)                                       \
     one((const void*)k_zcol_fwd<X>, X::kSmem);                 \
     one((const void*)k_zcol_inv<X>, X::kSmem);
+    switch (nz) {
 #define FLUSI_CASE(n, R, L)                                    \
-    {                                                          \
+    case n: {                                                  \
         using Full = Col<R, L, z_cols<n>()>;                   \
         using Small = Col<R, L, z_small<n>()>;                 \
         FLUSI_KERNELS(Full)                                    \
         FLUSI_KERNELS(Small)                                   \
+        break;                                                 \
     }
-    FLUSI_COL_LENGTHS(FLUSI_CASE)
+        FLUSI_COL_LENGTHS(FLUSI_CASE)
 #undef FLUSI_CASE
+    }
 #undef FLUSI_KERNELS
     return e;
 }

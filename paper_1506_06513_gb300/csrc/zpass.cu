@@ -968,8 +968,7 @@ cudaError_t launch_divergence(int fp64, const void* U, const Geom& g, unsigned l
 cudaError_t configure_zpass()
 {
     const int big = 120 * 1024;
-    cudaError_t e = configure_zcol();
-    if (e) return e;
+    cudaError_t e;
 #define FLUSI_SMEM(fn) \
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
 #define FLUSI_SMEM_Z(T, R16)                  \
