@@ -313,10 +313,12 @@ struct StepState {
 // kernel start (by the scalar kernel beside the forward passes, by a block whose
 // wait gave up), and a block that lost only some of its threads would go on with
 // tables and barriers those threads never set up.  Every thread calls it.
+// A kernel whose tables need nothing of the step's data may read the word first
+// (step_failed) and take the vote at the barrier behind the tables.
+__device__ __forceinline__ bool step_failed(const StepState* st) { return st && *(volatile const int*)&st->status != 0; }
 __device__ __forceinline__ bool block_leaves(const StepState* st, const int* err)
 {
-    const bool gone = (st && *(volatile const int*)&st->status != 0) || (err && *(volatile const int*)err != 0);
-    return __syncthreads_or(gone) != 0;
+    return __syncthreads_or(step_failed(st) || (err && *(volatile const int*)err != 0)) != 0;
 }
 
 // Coefficients of the current step, written by the scalar kernel and read by

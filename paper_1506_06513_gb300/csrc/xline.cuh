@@ -316,7 +316,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (block_leaves(st, nullptr)) return;
+    const bool failed = step_failed(st);
     constexpr int NT = 96, NW = 3;
     constexpr int R = X::R, L = X::L, G = X::G, NH = X::NH, CS = X::CS, LP = X::LP;
     constexpr int RB = G, NG = NW * G;         // rows of a tile, lane groups of the block
@@ -338,6 +338,7 @@ k_xline_phys(float2* __restrict__ W, Geom g, const double2* __restrict__ tw, XEx
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     X::tables(twx, tw, g.nx);
     load_frame_t<float>(Fs, ex.frame);
+    if (__syncthreads_or(failed)) return;
     const auto p = X::lane_of(lane);
     const float dxT = float(g.dx), dyT = float(g.dy), dzT = float(g.dz);
     const FrameT<float>& F = *Fs;

@@ -192,7 +192,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (block_leaves(st, nullptr)) return;
+    const bool failed = step_failed(st);
     constexpr bool kPhys = (MODE == XP_PHYS || MODE == XP_DUMP);
     const int RB = 1 << lgRB;
     const int NF = kPhys ? 6 : ex.ncomp;
@@ -217,7 +217,7 @@ k_xpass(cplx<T>* __restrict__ W, Geom g, FftPlan plan, const double2* __restrict
         for (int i = tid; i < kWarpsX * 36; i += kThreadsX) wacc[i] = 0.0;
         load_frame_t<T>(Fs, ex.frame);
     }
-    __syncthreads();
+    if (__syncthreads_or(failed)) return;
     for (int p = tid; p < nh; p += kThreadsX) ipos[spos[p]] = p;
     __syncthreads();
 
@@ -587,7 +587,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
         ex.frame = m.fr;
         ex.part = m.part;
     }
-    if (block_leaves(st, nullptr)) return;
+    const bool failed = step_failed(st);
     constexpr int L = sq_lanes<R, S>();    // lanes per line
     constexpr int RB = sq_rows<L>();
     constexpr int NH = sq_nh<R, S>();
@@ -629,6 +629,7 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
         tw2[q * L + (S == 2 ? (jj ^ q) : jj)] = twv((2 * jj * q) % nx);
     }
     load_frame_t<T>(Fs, ex.frame);
+    if (__syncthreads_or(failed)) return;
 
     const T dxT = T(g.dx), dyT = T(g.dy), dzT = T(g.dz);
     const FrameT<T>& F = *Fs;
