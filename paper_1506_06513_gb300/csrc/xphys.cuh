@@ -288,16 +288,16 @@ __device__ __forceinline__ void warp_sums12(const double* v, double* w, int lane
 // tree therefore runs in FP32 instructions on values of three parts, of which only
 // what lies some 70 bits below the largest is ever rounded; FP64 adds the parts and
 // everything above the warp.  x pass with a sphere of 0.3 box lengths at 256^3: FP64
-// tree 286 us, this one 245 (156 without a body; with two parts, 48 bits, 232).  Sums
+// tree 286 us, this one 244 (156 without a body; with two parts, 48 bits, 232).  Sums
 // kept per lane over a tile cost registers that the transforms need: 512^3 x pass
 // 1090 -> 1171 us.  Where a partial sum could leave the FP32 range, and
-// for infinities and NaN, the warp takes the FP64 tree.
+// for infinities, the warp takes the FP64 tree.
 __device__ __forceinline__ void warp_sums12(const float* v, double* w, int lane)
 {
-    float size = 0.0f;
+    float big[4];   // (a NaN is passed over here: it comes out as one either way)
 #pragma unroll
-    for (int k = 0; k < 12; ++k) size = __fadd_rn(size, fabsf(v[k]));
-    if (__any_sync(0xffffffffu, !(size < 0x1p120f))) {   // 32 lanes of less stay under 2^125
+    for (int k = 0; k < 4; ++k) big[k] = fmaxf(fmaxf(fabsf(v[3 * k]), fabsf(v[3 * k + 1])), fabsf(v[3 * k + 2]));
+    if (__any_sync(0xffffffffu, fmaxf(fmaxf(fmaxf(big[0], big[1]), big[2]), big[3]) >= 0x1p120f)) {   // 32 lanes of less stay under 2^125
         double d[12];
 #pragma unroll
         for (int k = 0; k < 12; ++k) d[k] = double(v[k]);
