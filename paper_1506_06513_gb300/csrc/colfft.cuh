@@ -14,8 +14,11 @@
 // The kernels are persistent: a block keeps its twiddle table and loops over
 // tiles, and as soon as pass 2 has read a tile the next one's copies go out into
 // its place.  Loads, not arithmetic, are what these passes wait for.
-//   Radices up to 18 leave registers for three blocks of 256 threads per SM, one
-//   tile each.
+//   Radices up to 18 run three blocks of 256 threads per SM, one tile each, at 80
+//   registers a thread: the y and forward z passes fit but for 24 bytes of spills
+//   at 324 rows; the inverse z pass, which holds side rows besides, spills 148 and
+//   128 bytes at 324 rows (8 and 16 columns), 56 and 120 at 288, 80 and 20 at 256
+//   (8 and 32), up to 28 at 162 to 216.  Two blocks per SM were not measured for it.
 //   Larger ones leave two groups of 256 threads, but shared memory for three
 //   tiles: they form one block of two groups over a ring of three tiles, each
 //   group taking every second load, so that one tile is always on its way (y
@@ -28,7 +31,8 @@
 //   is transformed): 5.1 and 4.3 ms, the forward passes 2.3 and 1.7 (z staged 2.8).
 
 // A tile's rows are C consecutive values, so a warp's 8-byte accesses cover whole
-// 128-byte lines (C >= 16); with C = 8 (n > 512) pass 2 meets each bank twice.
+// 128-byte lines (C >= 16); with C = 8 (the narrow z tile, up to 512 rows) pass 2
+// meets each bank twice.
 #pragma once
 
 #include "fft.cuh"
@@ -265,8 +269,10 @@ __device__ __forceinline__ void col_loop(float2* bufs, ColState& sh, bool tma, i
             if (sh.issued[b] > 0) mbar_wait(sh.full + b, (unsigned)(sh.issued[b] - 1) & 1u, limit);
 }
 
-// The lengths served, X(n, R, L).  Others (and narrowed tiles, the other plans
-// and FP64) take the staged kernels of ypass.cu and zpass.cu.
+// The lengths served, X(n, R, L): from 64 rows on all but 729 (the halves of a tile
+// over 512 rows need an even R) and 972 (no R, L up to 32).  Those, tiles narrowed
+// by y_cols or z_cols, the other plans and FP64 take the staged kernels of ypass.cu
+// and zpass.cu.
 #define FLUSI_COL_LENGTHS(X)                                                                               \
     X(64, 8, 8) X(72, 9, 8) X(81, 9, 9) X(96, 12, 8) X(108, 12, 9) X(128, 16, 8) X(144, 12, 12)            \
     X(162, 18, 9) X(192, 16, 12) X(216, 18, 12) X(243, 27, 9) X(256, 16, 16) X(288, 18, 16) X(324, 18, 18) \

@@ -43,9 +43,9 @@ __device__ __forceinline__ double2 caxpy(double s, double2 x, double2 a)
 // FP32 complex values as packed pairs (add/mul/fma.f32x2): one instruction
 // where the scalar forms take two, with the same rounding.  The FP32
 // transforms are bound by instruction issue, not by the FMA pipe (which a
-// packed instruction holds for two cycles): at 512^3 the x pass went from
-// 1.285 to 1.245 ms, the z inverse from 0.484 to 0.472, the y passes from
-// 0.692 and 0.337 to 0.682 and 0.321, the forward z pass from 0.228 to 0.213.
+// packed instruction holds for two cycles): alone, at 512^3, they took the x pass
+// from 1.285 to 1.245 ms and the staged y and z passes that ran there then from
+// 0.692, 0.337, 0.484 and 0.228 to 0.682, 0.321, 0.472 and 0.213.
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }

@@ -1,4 +1,4 @@
-// Small single-block kernels of one step:
+// Small kernels of one step, one warp (kinematics), one cluster (scalars), one thread (reset):
 //  * kinematics: the insect frames at t^n (Sec. 3.1, 3.3; Eq. M_body_yawpitchroll),
 //    in FP64, written as one Frame block read by every CTA of the physical pass;
 //  * scalars: the deterministic final reduction of the physical pass's per-CTA

@@ -22,11 +22,12 @@
 // What bounds it: shared-memory wavefronts and instruction issue, as for the
 // square kernels; the general shared-memory kernel (k_xpass) that served these
 // lengths goes through shared memory once per radix-8/4/3 stage.  Measured,
-// FP32, k_xpass -> these: physical pass 384 x 384 x 768 3.27 -> 1.35 ms (3.1 GB
-// of lines: 2.3 TB/s), 192^3 233 -> 93 us, 162 x 81 x 243 133 -> 49 us,
-// 48 x 36 x 24 33 -> 22 us; sponge lines 384 x 384 x 768 2.07 -> 0.58 ms;
-// set_state and get_state at 512^3 3.36 and 2.23 -> 1.32 and 1.04 ms, at
-// 1024^3 29.1 and 19.8 -> 13.0 and 9.7 ms (their z and y passes included).
+// FP32, k_xpass -> these: physical pass 384 x 384 x 768 3.27 -> 1.25 ms (3.1 GB
+// of lines: 2.5 TB/s), 192^3 233 -> 90 us, 162 x 81 x 243 133 -> 49 us,
+// 48 x 36 x 24 33 -> 18 us; sponge lines 384 x 384 x 768 2.07 -> 0.52 ms;
+// set_state and get_state at 512^3 3.36 and 2.23 -> 1.33 and 0.94 ms, at
+// 1024^3 29.1 and 19.8 -> 10.6 and 8.1 ms (their z and y passes included, which
+// became faster too).
 #pragma once
 
 #include "fft.cuh"

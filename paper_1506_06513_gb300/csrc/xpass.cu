@@ -13,8 +13,9 @@
 //   smoothing_mask_as_function_of_delta), u_s = u_b + Omega_w x (x - x_pivot)
 //   (Eqs. body_velocity_field, wing_velocity_field), and
 //   NL = u x omega - chi/C_eta (u - u_s)  (Eq. PNST_org_momentum),
-//   plus FP64 partial sums of chi (u - u_s), r x chi (u - u_s), chi u_s,
-//   r x chi u_s per colour, |u|^2, max |u|^2 and a non-finite flag.
+//   plus partial sums (a point's in the pass's precision, FP64 from the warp or, for
+//   |u|^2, the tile up) of chi (u - u_s), r x chi (u - u_s), chi u_s, r x chi u_s per
+//   colour, |u|^2, max |u|^2 and a non-finite flag.
 // The grid is persistent (a multiple of the SM count); each CTA writes one
 // row of partial sums, reduced in a fixed order by the scalar kernel.
 #include <algorithm>

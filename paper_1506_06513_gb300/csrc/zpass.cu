@@ -683,7 +683,8 @@ k_zupdate(const cplx<T>* __restrict__ Wn, cplx<T>* __restrict__ U, cplx<T>* __re
 
 // Whether the two-pass kernels run a grid's z passes: by the grid and its tuning
 // alone, whatever the batch, so that members equal solo runs bit for bit.  Over 512
-// rows they have one tile, taken where it fills the chip.
+// rows they have one tile, taken where it fills the GB300's SMs (a fixed number: the
+// staged kernels round differently).
 template <typename T> bool z_two_pass(const Geom& g)
 {
     const int full = sizeof(T) == 4 && g.two_pass_z ? zcol_full(g.nz) : 0;
