@@ -27,6 +27,9 @@
  *    in a device status word; they surface at the next call that synchronizes
  *    (flusi_forces, flusi_get_state, flusi_get_spectrum, flusi_sync), after
  *    which flusi_step returns FLUSI_ESTATE until the next flusi_set_state.
+ *    In FP32 at nx = 96, 512 and 1024 (64, 128 and 256 with the sponge) the
+ *    check is that of |u|^2: a term that overflows under a finite velocity is
+ *    reported a step later.
  */
 #ifndef FLUSI_H
 #define FLUSI_H

@@ -754,9 +754,9 @@ k_xpass_sq(cplx<T>* __restrict__ W, Geom g, const double2* __restrict__ tw, XExt
 
         // ---- physical space, every point: NL = u x omega into the omega lines,
         //      energy and max |u|^2.  A non-finite velocity makes the energy sum
-        //      non-finite; NL can only be non-finite through u (omega, u_s and
-        //      the penalization are finite for a finite state), so the energy
-        //      sum is the check.
+        //      non-finite, and the sum is the check.  (A product or a
+        //      penalization that overflows while u is finite, above 1e17 or so
+        //      in FP32, makes the next state non-finite and is reported then.)
         //      FP32 radix-16 and rectangular lines without the wake terms: two
         //      point pairs per thread (logical rows 2m, 2m + 1 sit in adjacent
         //      slots of those layouts), as 16-byte accesses.
