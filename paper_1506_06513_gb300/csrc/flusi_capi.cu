@@ -564,7 +564,7 @@ std::string flusi::tuning_key(flusi_t h)
         if (c == ' ' || c == '\t') c = '_';
     const bool wake = h->opt.sponge_c > 0 || h->opt.layer_width[0] > 0 || h->opt.layer_width[1] > 0 ||
                       h->opt.layer_width[2] > 0;
-    char buf[256];
+    char buf[512];
     std::snprintf(buf, sizeof buf, "%s|%d|%dx%dx%d|%s|%s|%s|d%d|%s", name.empty() ? "gpu" : name.c_str(),
                   prop.multiProcessorCount, h->nx, h->ny, h->nz,
                   h->prec == FLUSI_FP64 ? "fp64" : h->prec == FLUSI_FP32 ? "fp32" : h->prec == FLUSI_FP32_SPLITBF16 ? "bf16x2" : "bf16x3",
